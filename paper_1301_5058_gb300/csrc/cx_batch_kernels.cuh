@@ -134,9 +134,10 @@ template <typename T, int STAGE> constexpr int batch_min_blocks()
 template <typename T, int LAW, int MOB, int NOISE, int STAGE>
 __global__ void __launch_bounds__(kThreads, batch_min_blocks<T, STAGE>())
     batch_step_kernel(const InstDev<T> *__restrict__ inst, const int4 *__restrict__ work,
-                      int parity, int rows, const long long *__restrict__ step_base, int step_off)
+                      int parity, int rows, const long long *step_base, int step_off)
 {
-    const uint64_t step = NOISE ? (uint64_t)(__ldg(step_base) + step_off) : 0;
+    pass_wait();
+    const uint64_t step = NOISE ? (uint64_t)(*step_base + step_off) : 0;
     tile_step<T, LAW, MOB, NOISE, STAGE, false>(inst, work[blockIdx.x], parity, rows, step);
 }
 
@@ -151,18 +152,20 @@ template <typename T> constexpr int batch_fused_min_blocks() { return sizeof(T) 
 template <typename T, int LAW, int MOB, int NOISE, bool HEUN>
 __global__ void __launch_bounds__(kBatchFusedThreads, batch_fused_min_blocks<T>())
     batch_fused_kernel(const InstDev<T> *__restrict__ inst, const int4 *__restrict__ work,
-                       int parity, int rows, const long long *__restrict__ step_base, int step_off)
+                       int parity, int rows, const long long *step_base, int step_off)
 {
+    // the tables are not written while a pass may be queued
     const int4 w = work[blockIdx.x];
     const InstDev<T> &I = inst[w.x];
     const int nx = I.nx, ny = I.ny;
     const long long pitch = I.pitch;
     const KV<P2<T>> k = make_kv(I.k);
+    pass_wait();
     const Ptrs<T> P{I.b[parity], I.n[parity], I.s, nullptr, nullptr, I.b[parity ^ 1],
                     I.n[parity ^ 1]};
     // NOISE 1: stage one draws sigma for the pass's first step; Euler's
     // second stage for the next step, Heun's second stage shares the first's
-    const uint64_t step = NOISE ? (uint64_t)(__ldg(step_base) + step_off) : 0;
+    const uint64_t step = NOISE ? (uint64_t)(*step_base + step_off) : 0;
     const NoiseT<T> nz1 = NOISE ? inst_noise(I, step) : NoiseT<T>{};
     const NoiseT<T> nz2 = NOISE && !HEUN ? inst_noise(I, step + 1) : nz1;
     const int lane = threadIdx.x & 31;
@@ -191,12 +194,10 @@ cudaError_t launch_step_n(const void *inst, const int4 *work, int nwork, int par
 {
     const InstDev<T> *ip = (const InstDev<T> *)inst;
     if (stage == 0)
-        batch_step_kernel<T, LAW, MOB, NOISE, 0><<<nwork, kThreads, 0, st>>>(ip, work, parity, rows,
-                                                                             step_base, step_off);
-    else
-        batch_step_kernel<T, LAW, MOB, NOISE, 1><<<nwork, kThreads, 0, st>>>(ip, work, parity, rows,
-                                                                             step_base, step_off);
-    return cudaGetLastError();
+        return launch_pass(batch_step_kernel<T, LAW, MOB, NOISE, 0>, nwork, kThreads, 0, st, ip, work,
+                           parity, rows, step_base, step_off);
+    return launch_pass(batch_step_kernel<T, LAW, MOB, NOISE, 1>, nwork, kThreads, 0, st, ip, work,
+                       parity, rows, step_base, step_off);
 }
 
 template <typename T, int LAW, int MOB>
@@ -215,12 +216,10 @@ cudaError_t launch_fused_n(const void *inst, const int4 *work, int nwork, int pa
 {
     const InstDev<T> *ip = (const InstDev<T> *)inst;
     if (heun)
-        batch_fused_kernel<T, LAW, MOB, NOISE, true><<<nwork, kBatchFusedThreads, 0, st>>>(
-            ip, work, parity, rows, step_base, step_off);
-    else
-        batch_fused_kernel<T, LAW, MOB, NOISE, false><<<nwork, kBatchFusedThreads, 0, st>>>(
-            ip, work, parity, rows, step_base, step_off);
-    return cudaGetLastError();
+        return launch_pass(batch_fused_kernel<T, LAW, MOB, NOISE, true>, nwork, kBatchFusedThreads, 0,
+                           st, ip, work, parity, rows, step_base, step_off);
+    return launch_pass(batch_fused_kernel<T, LAW, MOB, NOISE, false>, nwork, kBatchFusedThreads, 0, st,
+                       ip, work, parity, rows, step_base, step_off);
 }
 
 template <typename T, int LAW, int MOB>

@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(fused_threads<NOISE>(),
     fused_kernel(Ptrs<T> P, int nx, int ny, long long pitch, KV<P2<T>> k, NoiseT<T> nz1,
                  NoiseT<T> nz2, int rows)
 {
+    pass_wait();
     constexpr int kBlockCols = (fused_threads<NOISE>() / 32) * kFusedCols;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int xb = blockIdx.x * kBlockCols;  // first written column of the block
@@ -77,12 +78,10 @@ cudaError_t launch_t(const StepArgs &a, cudaStream_t st)
     const dim3 grid((a.nx + cols - 1) / cols, (a.ny + a.rows - 1) / a.rows);
     // 32-bit element offsets for the per-step passes when every offset fits
     if (NOISE == 1 && (long long)a.ny * a.pitch < (1LL << 31))
-        fused_kernel<T, LAW, MOB, NOISE, HEUN, NOISE == 1><<<grid, threads, 0, st>>>(
-            P, a.nx, a.ny, a.pitch, k, nz1, nz2, a.rows);
-    else
-        fused_kernel<T, LAW, MOB, NOISE, HEUN, false><<<grid, threads, 0, st>>>(
-            P, a.nx, a.ny, a.pitch, k, nz1, nz2, a.rows);
-    return cudaGetLastError();
+        return launch_pass(fused_kernel<T, LAW, MOB, NOISE, HEUN, NOISE == 1>, grid, threads, 0, st,
+                           P, a.nx, a.ny, a.pitch, k, nz1, nz2, a.rows);
+    return launch_pass(fused_kernel<T, LAW, MOB, NOISE, HEUN, false>, grid, threads, 0, st, P, a.nx,
+                       a.ny, a.pitch, k, nz1, nz2, a.rows);
 }
 
 // One (precision, law, mobility) combination: every noise mode and scheme.

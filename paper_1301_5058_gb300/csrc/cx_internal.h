@@ -19,6 +19,39 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// Launches a pass kernel as a programmatic dependent of the kernel before it
+// in the stream: the launch is set up while that kernel drains, and the
+// kernel's blocks wait in pass_wait() for its writes instead of being launched
+// after them.  A chain of small passes then costs 1.5 instead of 4.1 us per
+// pass on its own (152 empty blocks), and a pass 2.3 us less: 64^2 2.7 -> 1.5,
+// 256^2 4.1 -> 2.7, 1024^2 5.1 -> 4.3, 2048^2 11.3 -> 9.9 us per time step.
+// The kernels do not release their dependents early
+// (cudaTriggerProgrammaticLaunchCompletion): the next pass's blocks would then
+// fill the first SMs that drain two deep and leave others empty (256^2 in FP64
+// 20.7 -> 30.2 us per step, 2048^2 in FP32 9.9 -> 10.7).
+template <typename... P, typename... A>
+inline cudaError_t launch_pass(void (*kern)(P...), dim3 grid, int threads, size_t smem,
+                               cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, P(args)...);
+}
+#ifdef __CUDACC__
+// Every kernel launched by launch_pass calls this before it reads or writes
+// what other kernels of the stream write or read.  What comes after is loaded
+// coherently (no __ldg, whose loads the compiler may move ahead of this).
+__device__ __forceinline__ void pass_wait() { cudaGridDependencySynchronize(); }
+#endif
+
 // Per-run coefficients of the face fluxes.  The kernels evaluate unscaled
 // face fluxes and apply the constant factors once per cell, so that one
 // step reads

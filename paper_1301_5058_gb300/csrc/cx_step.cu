@@ -45,6 +45,7 @@ template <typename T, int LAW, int MOB, int NOISE, int STAGE>
 __global__ void __launch_bounds__(kThreads, step_min_blocks<T, NOISE, STAGE>())
     step_kernel(Ptrs<T> P, int nx, int ny, long long pitch, KV<P2<T>> k, NoiseT<T> nz, int rows)
 {
+    pass_wait();
     const int x0 = (blockIdx.x * kThreads + threadIdx.x) * kCells;
     const int j0 = blockIdx.y * rows;
     const int jend = min(j0 + rows, ny);
@@ -78,9 +79,8 @@ cudaError_t launch_t(const StepArgs &a, cudaStream_t st)
               (const T *)a.nu, (T *)a.bo, (T *)a.no};
     const dim3 grid((a.nx + kThreads * kCells - 1) / (kThreads * kCells),
                     (a.ny + a.rows - 1) / a.rows);
-    step_kernel<T, LAW, MOB, NOISE, STAGE><<<grid, kThreads, 0, st>>>(P, a.nx, a.ny, a.pitch, k, nz,
-                                                                        a.rows);
-    return cudaGetLastError();
+    return launch_pass(step_kernel<T, LAW, MOB, NOISE, STAGE>, grid, kThreads, 0, st, P, a.nx, a.ny,
+                       a.pitch, k, nz, a.rows);
 }
 
 template <typename T, int LAW, int MOB>
