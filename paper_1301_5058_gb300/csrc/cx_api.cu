@@ -249,7 +249,13 @@ cx::Coef cx::make_coef(const cx_grid &g, const cx_params &p, double dt)
     const double dx2 = g.dx * g.dx;
     cx::Coef k;
     k.cA = dt / (8.0 * dx2);
-    k.cChi = p.chemo_law == CX_CHEMO_RECEPTOR ? 2.0 * p.chi0 : 0.5 * p.chi0;
+    const bool donor = p.mobility == CX_MOBILITY_UPWIND;
+    if (p.chemo_law == CX_CHEMO_RECEPTOR && p.precision == CX_PREC_F64)
+        k.cChi = fmin((donor ? 0.5 : 1.0) / sqrt(2.0 * p.chi0), cx::kNoChemoF64);
+    else if (p.chemo_law == CX_CHEMO_RECEPTOR)
+        k.cChi = (donor ? 8.0 : 2.0) * p.chi0;
+    else
+        k.cChi = (donor ? 2.0 : 0.5) * p.chi0;
     k.cG = dt * p.Dn / dx2;
     k.cR = dt * p.theta;
     k.cN = dt;
@@ -325,8 +331,31 @@ int cx_dt_limit(const cx_grid *g, const cx_params *p, double *limit)
 // sides 512, 1024, 1536 and 2048, the fastest measured heights or within
 // 4 % of them (the earlier 480-column estimate picked 1, 3, 6 and 9 rows,
 // 18-49 % slower), and 64 rows at 16384^2.
+//
+// FP64, one stage per pass: one-warp blocks of 128 columns, bound by the FP64
+// units, one per scheduler (four per SM).  A block of r rows costs about
+// r + 1/2 rows (it evaluates the y-faces behind its first row again), so the
+// height taken is the one with the least ceil(blocks / units) (r + 1/2).
+static int auto_tile_rows_f64(const cx_ctx *c)
+{
+    const long long tiles_x = ((long long)c->g.nx + 127) / 128, units = 4LL * c->num_sms;
+    long long best = 1;
+    double cost = 0.0;
+    for (long long r = 1; r <= 32; ++r) {
+        const long long tiles_y = ((long long)c->g.ny + r - 1) / r;
+        if (tiles_y > 65535) continue;
+        const double now = (double)((tiles_x * tiles_y + units - 1) / units) * ((double)r + 0.5);
+        if (cost == 0.0 || now <= cost) {
+            cost = now;
+            best = r;
+        }
+    }
+    return (int)best;
+}
+
 static int auto_tile_rows(const cx_ctx *c)
 {
+    if (c->prec == CX_PREC_F64 && c->time_block == 1) return auto_tile_rows_f64(c);
     const bool two = c->time_block == 2;
     const bool one_warp = two && c->p.noise_mode != CX_NOISE_PER_STEP;
     const long long cols = !two ? 512 : one_warp ? 120 : 480;

@@ -196,7 +196,7 @@ void fill_inst(int prec, void *table, int i, void *b0, void *b1, void *n0, void 
         d.b[0] = (double *)b0; d.b[1] = (double *)b1; d.n[0] = (double *)n0; d.n[1] = (double *)n1;
         d.s = (const double *)s;
         d.nx = nx; d.ny = ny; d.pitch = pitch;
-        d.k = CoefT<double>{k.cA, k.cChi, k.cG, k.cR, k.cN};
+        d.k = stencil::coef_t<double>(k);
         d.fth = reduce::float_threshold(bth);
         d.bth = bth;
         d.seed = seed;
@@ -208,7 +208,7 @@ void fill_inst(int prec, void *table, int i, void *b0, void *b1, void *n0, void 
         d.b[0] = (float *)b0; d.b[1] = (float *)b1; d.n[0] = (float *)n0; d.n[1] = (float *)n1;
         d.s = (const float *)s;
         d.nx = nx; d.ny = ny; d.pitch = pitch;
-        d.k = CoefT<float>{(float)k.cA, (float)k.cChi, (float)k.cG, (float)k.cR, (float)k.cN};
+        d.k = stencil::coef_t<float>(k);
         d.fth = reduce::float_threshold(bth);
         d.bth = bth;
         d.seed = seed;

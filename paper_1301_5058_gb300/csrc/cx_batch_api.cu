@@ -27,7 +27,8 @@ int bcuda(cudaError_t e, const char *what)
         if (e_ != cudaSuccess) return bcuda(e_, (what));     \
     } while (0)
 
-constexpr int kTileCols = 512;       // columns per tile (128 threads x 4 cells)
+// columns per tile of the one-stage march: 128 threads (FP32) or 32 (FP64) x 4 cells
+int tile_cols(int prec) { return prec == CX_PREC_F64 ? 128 : 512; }
 constexpr int kFusedTileCols = 120;  // written columns per (one-warp) tile of the two-stage march
 constexpr int kDiagBlocksPerInst = 64;
 
@@ -50,7 +51,7 @@ struct cx_batch {
     size_t elem = 4;
     void *d_inst = nullptr;
     std::vector<unsigned char> h_inst;
-    int4 *d_work = nullptr;       // 512-column tiles (one stage per pass)
+    int4 *d_work = nullptr;       // tile_cols() tiles (one stage per pass)
     std::vector<int> work_begin;  // first work item of each instance (+ total)
     int4 *d_work2 = nullptr;      // 120-column tiles (two stages per pass)
     std::vector<int> work2_begin;
@@ -102,12 +103,12 @@ void free_batch(cx_batch *B)
 }
 
 // Tile work lists for the current tile height, instance by instance: the
-// one-stage march's 512-column tiles and the two-stage march's 120-column
+// one-stage march's tiles and the two-stage march's 120-column
 // tiles.
 int build_work(cx_batch *B)
 {
     for (int f = 0; f < 2; ++f) {
-        const int cols = f ? kFusedTileCols : kTileCols;
+        const int cols = f ? kFusedTileCols : tile_cols(B->prec);
         std::vector<int> &begin = f ? B->work2_begin : B->work_begin;
         int4 *&d = f ? B->d_work2 : B->d_work;
         std::vector<int4> w;

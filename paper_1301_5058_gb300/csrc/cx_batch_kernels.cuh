@@ -34,10 +34,11 @@ __device__ __forceinline__ void tile_step(const InstDev<T> *__restrict__ inst, c
                     I.b[parity], I.n[parity]};
     }
     const NoiseT<T> nz = NOISE ? inst_noise(I, step) : NoiseT<T>{};
-    const int x0 = (w.y * kThreads + threadIdx.x) * kCells;
+    constexpr int kTileCols = step_threads<T>() * kCells;
+    const int x0 = w.y * kTileCols + threadIdx.x * kCells;
     const int j0 = w.z * rows;
     const int jend = min(j0 + rows, ny);
-    const bool interior = w.y > 0 && (w.y + 1) * kThreads * kCells < nx;
+    const bool interior = w.y > 0 && (w.y + 1) * kTileCols < nx;
     if (w.z & 1) {
         if (interior)
             march<T, LAW, MOB, NOISE, STAGE, -1, CG, true>(P, nx, ny, pitch, k, nz, x0, j0, jend);
@@ -92,16 +93,16 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier *gb, long long spin_lim
 // Several steps of a group of instances in one cooperative launch: the
 // group's tiles are dealt to the resident blocks, and a grid barrier
 // separates the steps (and Heun's stages).  Loads go through L2 only.
-// Register budget: 2 blocks per SM (the launch sizes its grid from the
+// Register budget: 2 four-warp or 8 one-warp blocks per SM (the launch sizes its grid from the
 // occupancy this leaves).  The kernel inlines every march variant; its FP64
 // Heun forms still spill a little at 255 registers.
-template <typename T> constexpr int resident_min_blocks() { return 2; }
+template <typename T> constexpr int resident_min_blocks() { return sizeof(T) == 4 ? 2 : 8; }
 
 // The time step of the first pass of a launch is *step_base + step_off:
 // the host writes step_base before a captured graph is replayed, and the
 // passes inside the graph add their fixed offsets (read only with NOISE 1).
 template <typename T, int LAW, int MOB, int NOISE, int HEUN>
-__global__ void __launch_bounds__(kThreads, resident_min_blocks<T>())
+__global__ void __launch_bounds__(step_threads<T>(), resident_min_blocks<T>())
     batch_resident_kernel(const InstDev<T> *__restrict__ inst, const int4 *__restrict__ work,
                           int nwork, int parity, int rows, int nsteps, GridBarrier *gb,
                           long long spin_limit, const long long *__restrict__ step_base,
@@ -125,14 +126,15 @@ __global__ void __launch_bounds__(kThreads, resident_min_blocks<T>())
 // stage 0: u_out(parity^1) = u(parity) + dt r(u(parity))
 // stage 1: u(parity) = (u(parity) + u*(parity^1) + dt r(u*)) / 2, in place
 // As the single-grid step kernel: FP32 Euler steps are bound by HBM
-// bandwidth (64 registers, 8 blocks per SM); Heun's second stage 4; FP64 2.
+// bandwidth (64 registers, 8 blocks per SM); Heun's second stage 4; FP64 8
+// one-warp blocks.
 template <typename T, int STAGE> constexpr int batch_min_blocks()
 {
-    return sizeof(T) == 4 ? (STAGE == 0 ? 8 : 4) : 2;
+    return sizeof(T) == 4 ? (STAGE == 0 ? 8 : 4) : 8;
 }
 
 template <typename T, int LAW, int MOB, int NOISE, int STAGE>
-__global__ void __launch_bounds__(kThreads, batch_min_blocks<T, STAGE>())
+__global__ void __launch_bounds__(step_threads<T>(), batch_min_blocks<T, STAGE>())
     batch_step_kernel(const InstDev<T> *__restrict__ inst, const int4 *__restrict__ work,
                       int parity, int rows, const long long *step_base, int step_off)
 {
@@ -194,9 +196,9 @@ cudaError_t launch_step_n(const void *inst, const int4 *work, int nwork, int par
 {
     const InstDev<T> *ip = (const InstDev<T> *)inst;
     if (stage == 0)
-        return launch_pass(batch_step_kernel<T, LAW, MOB, NOISE, 0>, nwork, kThreads, 0, st, ip, work,
-                           parity, rows, step_base, step_off);
-    return launch_pass(batch_step_kernel<T, LAW, MOB, NOISE, 1>, nwork, kThreads, 0, st, ip, work,
+        return launch_pass(batch_step_kernel<T, LAW, MOB, NOISE, 0>, nwork, step_threads<T>(), 0, st, ip,
+                           work, parity, rows, step_base, step_off);
+    return launch_pass(batch_step_kernel<T, LAW, MOB, NOISE, 1>, nwork, step_threads<T>(), 0, st, ip, work,
                        parity, rows, step_base, step_off);
 }
 
@@ -244,7 +246,7 @@ cudaError_t launch_resident_h(const void *inst, const int4 *work, int nwork, int
     const void *kern = (const void *)batch_resident_kernel<T, LAW, MOB, NOISE, HEUN>;
     int per_sm = 0, dev = 0, sms = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, batch_resident_kernel<T, LAW, MOB, NOISE, HEUN>, kThreads, 0);
+        &per_sm, batch_resident_kernel<T, LAW, MOB, NOISE, HEUN>, step_threads<T>(), 0);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
@@ -256,7 +258,7 @@ cudaError_t launch_resident_h(const void *inst, const int4 *work, int nwork, int
     void *args[] = {(void *)&ip, (void *)&work, (void *)&nwork, (void *)&parity, (void *)&rows,
                     (void *)&nsteps, (void *)&gp, (void *)&spin, (void *)&step_base,
                     (void *)&step_off};
-    return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kThreads), args, 0, st);
+    return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(step_threads<T>()), args, 0, st);
 }
 
 template <typename T, int LAW, int MOB>

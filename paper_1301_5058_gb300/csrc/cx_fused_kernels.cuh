@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(fused_threads<NOISE>(),
 template <typename T, int LAW, int MOB, int NOISE, bool HEUN>
 cudaError_t launch_t(const StepArgs &a, cudaStream_t st)
 {
-    const KV<P2<T>> k = make_kv(CoefT<T>{(T)a.k.cA, (T)a.k.cChi, (T)a.k.cG, (T)a.k.cR, (T)a.k.cN});
+    const KV<P2<T>> k = make_kv(coef_t<T>(a.k));
     NoiseT<T> nz1;
     nz1.seed = a.sg.seed;
     nz1.step = (uint64_t)a.step;

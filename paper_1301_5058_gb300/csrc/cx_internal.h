@@ -56,22 +56,28 @@ __device__ __forceinline__ void pass_wait() { cudaGridDependencySynchronize(); }
 // face fluxes and apply the constant factors once per cell, so that one
 // step reads
 //   b' = b + dt theta n b + cA (phiE - phiW + phiN - phiS)
-//   n' = n - dt n b       + cG (gE - gW + gN - gS)
+//   n' = n - dt n b       - cG (gE - gW + gN - gS)
 // with, on a face between L (left/lower) and R (right/upper),
-//   hc  = chi(n_f) / 2 = cChi / (2+n2)^2 (receptor law) or cChi (constant law)
-//   phi = s2 n2 b2 (db - hc b2 dn)                   central mobility b_f^2
-//   phi = s2 n2 (b2 db - 4 hc b_d^2 dn)              donor-cell mobility b_d^2
-//   g   = dn
-// where s2 = sL+sR, n2 = nL+nR, b2 = bL+bR, db = bR-bL, dn = nR-nL and b_d
-// is b of the lower-n cell.  Derivation: sigma_f n_f b_f = s2 n2 b2 / 8,
-// b_f^2 = b2^2 / 4 and, for the receptor law, chi(n_f) = 4 chi0 / (2+n2)^2.
+//   phi = s2 n2 b2 (db + hc b2 dm)          central mobility b_f^2
+//   phi = s2 n2 (b2 db + hc b_d^2 dm)       donor-cell mobility b_d^2
+//   g   = dm
+// where s2 = sL+sR, n2 = nL+nR, b2 = bL+bR, db = bR-bL, dm = nL-nR and b_d
+// is b of the lower-n cell.  hc = cChi under the constant law and, under the
+// receptor law, cChi / (2+n2)^2 in FP32 and 1 / (cChi (2+n2))^2 in FP64.  Derivation: sigma_f n_f b_f =
+// s2 n2 b2 / 8, b_f^2 = b2^2 / 4, so hc = chi(n_f) / 2 (central) or 2 chi(n_f)
+// (donor cell), and for the receptor law chi(n_f) = 4 chi0 / (2+n2)^2.
 struct Coef {
     double cA;    // dt / (8 dx^2)
-    double cChi;  // receptor: 2 chi0; constant: chi0 / 2
+    double cChi;  // constant: chi0 / 2; receptor: 2 chi0; donor cell: 4 times
+                  // that.  Receptor in FP64: 1 / sqrt of it (kNoChemoF64 at most)
     double cG;    // dt Dn / dx^2
     double cR;    // dt theta
     double cN;    // dt
 };
+
+// The FP64 receptor law's scale without chemotaxis: the weight is then 2^-1002,
+// below the rounding of any flux (and the square of the denominator is finite).
+constexpr double kNoChemoF64 = 0x1p500;
 
 struct Sigma {  // how sigma is obtained
     int per_step;     // 0: read the sigma array; 1: regenerate from Philox every step

@@ -3,6 +3,8 @@
 // scaled scheme, per-step noise, and the row march (see cx_step.cu).
 #pragma once
 
+#include <type_traits>
+
 #include "cx_internal.h"
 #include "cx_philox.cuh"
 
@@ -11,6 +13,13 @@ namespace stencil {
 
 
 constexpr int kThreads = 128;  // 4 warps side by side along x
+// Threads of a block of the one-stage march: one warp in FP64.  Its warps share
+// nothing; a warp's FP64 instruction holds its scheduler's FP64 unit for 64
+// cycles, so what counts is that every scheduler gets the same number of warp
+// rows, and blocks of 128 columns cut a grid finer than blocks of 512 (with the
+// faces evaluated once and the heights chosen for it, 256^2 18.7 -> 10.4 us per
+// step, 1024^2 113.4 -> 92.7, 4096^2 1477 -> 1304).
+template <typename T> constexpr int step_threads() { return sizeof(T) == 4 ? kThreads : 32; }
 constexpr int kCells = 4;      // cells per thread along x
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -26,6 +35,12 @@ template <> struct Vec<float> {
         asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
                      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
                      : "l"(p));
+    }
+    static __device__ __forceinline__ float load1(const float *p)
+    {
+        float v;
+        asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+        return v;
     }
     // L2 path (bypasses L1): for a persistent launch, where the arrays a
     // block reads were written by other blocks earlier in the same launch
@@ -44,6 +59,12 @@ template <> struct Vec<double> {
     {
         asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "l"(p));
         asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "l"(p + 2));
+    }
+    static __device__ __forceinline__ double load1(const double *p)
+    {
+        double v;
+        asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+        return v;
     }
     static __device__ __forceinline__ void load_cg(const double *p, double (&v)[4])
     {
@@ -101,55 +122,44 @@ __device__ __forceinline__ double2 sub_rn(double2 a, double2 b, double2)
 {
     return make_double2(__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y));
 }
-// c / q for the receptor-law weight (q = (2 + n_L + n_R)^2 >= 4).  FP32: c
-// times the hardware's approximate reciprocal (the FP32 path is judged by
-// tolerance).  rcp.approx.ftz and an explicit multiply, not __fdividef: q lies
-// nowhere near the ends of the FP32 range, and the range handling around
-// __fdividef (scalings of numerator and denominator, predicated off for every
-// such q but issued all the same) was a quarter of the march's instructions.
-// Same bits; 16384^2 two-stage pass 0.919 -> 0.847 ms, which is 0.94 of the
-// measured HBM bandwidth and no longer bound by instruction issue; paper's
-// scheme 1.226 -> 1.133 ms; 2048^2 12.3 -> 11.3 and 45.6 -> 39.4 us per step.
-// FP64: c times a
-// reciprocal refined by Newton's method for 1/q, x <- x + x (1 - q x), whose
-// relative error e becomes e^2 per step, from the hardware's approximate
-// FP64 reciprocal (rcp.approx.ftz.f64; q is never subnormal).  Any seed within
-// 2^-14 of 1/q is below FP64 rounding after the two steps (2^-28, then
-// 2^-56), so the weight is within about one ulp of c / q; the seed needs no
-// FP64 <-> FP32 conversions, which run on GB300's narrow FP64 pipe.
+// 1 / q for the receptor-law weight.  FP32: the hardware's approximate
+// reciprocal (the FP32 path is judged by tolerance).  rcp.approx.ftz, not
+// __fdividef: the range handling around __fdividef (scalings of numerator and
+// denominator, predicated off for every q that occurs but issued all the same)
+// was a quarter of the march's instructions.  16384^2 two-stage pass
+// 0.919 -> 0.847 ms, which is 0.94 of the measured HBM bandwidth and no longer
+// bound by instruction issue; paper's scheme 1.226 -> 1.133 ms; 2048^2
+// 12.3 -> 11.3 and 45.6 -> 39.4 us per step.
+// FP64: the hardware's approximate FP64 reciprocal x (rcp.approx.ftz.f64; q is
+// never subnormal) and one third-order correction: with e = 1 - q x,
+// 1 / q = x / (1 - e) = x (1 + e + e^2 + ...), so x + x (e + e^2) is off by
+// e^3, far below FP64 rounding for any seed within 2^-19.  Three operations on
+// GB300's narrow FP64 pipe where two Newton steps took four.
 __device__ __forceinline__ float rcp_w(float q)
 {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
     return r;
 }
-__device__ __forceinline__ float div_w(float c, float q) { return __fmul_rn(c, rcp_w(q)); }
-__device__ __forceinline__ double div_w(double c, double q)
+__device__ __forceinline__ double rcp_w(double q)
 {
     double x;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(q));
-    x = __fma_rn(x, __fma_rn(-q, x, 1.0), x);
-    x = __fma_rn(x, __fma_rn(-q, x, 1.0), x);
-    return __dmul_rn(c, x);
+    const double e = __fma_rn(-q, x, 1.0);
+    return __fma_rn(x, __fma_rn(e, e, e), x);
 }
-__device__ __forceinline__ float2 div_w(float2 c, float2 q)
+__device__ __forceinline__ float2 rcp_w(float2 q) { return make_float2(rcp_w(q.x), rcp_w(q.y)); }
+__device__ __forceinline__ double2 rcp_w(double2 q) { return make_double2(rcp_w(q.x), rcp_w(q.y)); }
+// donor-cell b: the side with the lower n (dm = nL - nR)
+__device__ __forceinline__ float donor(float dm, float bL, float bR) { return dm <= 0.f ? bL : bR; }
+__device__ __forceinline__ double donor(double dm, double bL, double bR) { return dm <= 0.0 ? bL : bR; }
+__device__ __forceinline__ float2 donor(float2 dm, float2 bL, float2 bR)
 {
-    return __fmul2_rn(c, make_float2(rcp_w(q.x), rcp_w(q.y)));
+    return make_float2(donor(dm.x, bL.x, bR.x), donor(dm.y, bL.y, bR.y));
 }
-__device__ __forceinline__ double2 div_w(double2 c, double2 q)
+__device__ __forceinline__ double2 donor(double2 dm, double2 bL, double2 bR)
 {
-    return make_double2(div_w(c.x, q.x), div_w(c.y, q.y));
-}
-// donor-cell b: the side with the lower n (dn = nR - nL)
-__device__ __forceinline__ float donor(float dn, float bL, float bR) { return dn >= 0.f ? bL : bR; }
-__device__ __forceinline__ double donor(double dn, double bL, double bR) { return dn >= 0.0 ? bL : bR; }
-__device__ __forceinline__ float2 donor(float2 dn, float2 bL, float2 bR)
-{
-    return make_float2(donor(dn.x, bL.x, bR.x), donor(dn.y, bL.y, bR.y));
-}
-__device__ __forceinline__ double2 donor(double2 dn, double2 bL, double2 bR)
-{
-    return make_double2(donor(dn.x, bL.x, bR.x), donor(dn.y, bL.y, bR.y));
+    return make_double2(donor(dm.x, bL.x, bR.x), donor(dm.y, bL.y, bR.y));
 }
 __host__ __device__ __forceinline__ float2 pair(float x, float y) { return make_float2(x, y); }
 __host__ __device__ __forceinline__ double2 pair(double x, double y) { return make_double2(x, y); }
@@ -158,65 +168,90 @@ __host__ __device__ __forceinline__ double2 pair(double x, double y) { return ma
 template <typename T> struct CoefT {
     T cA, cChi, cG, cR, cN;
 };
+template <typename T> CoefT<T> coef_t(const Coef &k)
+{
+    return CoefT<T>{(T)k.cA, (T)k.cChi, (T)k.cG, (T)k.cR, (T)k.cN};
+}
 
 // The coefficients and constants of the face and update arithmetic, for
 // one cell (V = T) or a pair (V = P2<T>): signs are folded in so that every
 // subtraction of a product is one multiply-add.
 template <typename V> struct KV {
     V cA;     // scale of the bacterial flux divergence
-    V ncChi;  // -chi0 scale
-    V cG;     // scale of the nutrient flux divergence
+    V chi;    // constant law: hc; receptor law: FP32 its numerator, FP64 the scale of q
+    V two;    // receptor law: FP32 2, FP64 twice chi
+    V ncG;    // -scale of the nutrient flux divergence
     V cR;     // growth
     V ncN;    // -consumption
-    V two, four, m1, half;
+    V m1, half;
 };
 template <typename T> __host__ __device__ __forceinline__ KV<P2<T>> make_kv(const CoefT<T> &k)
 {
     KV<P2<T>> v;
     v.cA = pair(k.cA, k.cA);
-    v.ncChi = pair(-k.cChi, -k.cChi);
-    v.cG = pair(k.cG, k.cG);
+    v.chi = pair(k.cChi, k.cChi);
+    v.two = sizeof(T) == 4 ? pair(T(2), T(2)) : pair(T(2) * k.cChi, T(2) * k.cChi);
+    v.ncG = pair(-k.cG, -k.cG);
     v.cR = pair(k.cR, k.cR);
     v.ncN = pair(-k.cN, -k.cN);
-    v.two = pair(T(2), T(2));
-    v.four = pair(T(4), T(4));
     v.m1 = pair(T(-1), T(-1));
     v.half = pair(T(0.5), T(0.5));
     return v;
 }
 template <typename T> __device__ __forceinline__ KV<T> scalar_kv(const KV<P2<T>> &k)
 {
-    return KV<T>{k.cA.x, k.ncChi.x, k.cG.x, k.cR.x, k.ncN.x, k.two.x, k.four.x, k.m1.x, k.half.x};
+    return KV<T>{k.cA.x, k.chi.x, k.two.x, k.ncG.x, k.cR.x, k.ncN.x, k.m1.x, k.half.x};
+}
+
+// The receptor law's weight at a face (see face()).
+template <typename V> __device__ __forceinline__ V weight(V n2, const KV<V> &k)
+{
+    if constexpr (std::is_same<V, float>::value || std::is_same<V, float2>::value) {
+        const V q = add_rn(n2, k.two);
+        return mul_rn(k.chi, rcp_w(mul_rn(q, q)));
+    } else {
+        const V q = fma_rn(n2, k.chi, k.two);
+        return rcp_w(mul_rn(q, q));
+    }
 }
 
 // Unscaled fluxes (phi, g) through the face between L (left/lower) and R,
 // for one face or a pair of faces:
-//   phi = s2 n2 b2 (db - hc b2 dn)          (central b^2 mobility)
-//   phi = s2 n2 (b2 db - 4 hc bd^2 dn)       (donor-cell b^2)
-//   g   = dn
-// with s2 = sL + sR (likewise n2, b2), db = bR - bL, dn = nR - nL and
-// hc = cChi / (2 + n2)^2 (receptor law) or cChi (constant chi).  The
-// constant factors cA and cG are applied once per cell, to the divergence
-// (cell_update), not once per face.
+//   phi = s2 n2 b2 (db + hc b2 dm)      (central b^2 mobility)
+//   phi = s2 n2 (b2 db + hc bd^2 dm)    (donor-cell b^2)
+//   g   = dm
+// with s2 = sL + sR (likewise n2, b2), db = bR - bL, dm = nL - nR and, under
+// the constant law, hc = chi.  The receptor law's weight is in FP32
+// hc = chi / (2 + n2)^2.  In FP64 its strength is folded into the scale of the
+// denominator, hc = 1 / q^2 with q = chi n2 + 2 chi, so that no face multiplies
+// by it: the FP64 kernels are bound by the FP64 pipe and take 15 operations per
+// face instead of 17 (with rcp_w), 4096^2 1630 -> 1476 us per step, 1024^2
+// 125.6 -> 113.4.  In FP32 the second constant of that multiply-add costs the
+// marches a register pair that they do not have (16384^2 422 -> 428 us per
+// step, the paper's scheme 1118 -> 1171).  The constant factors cA and cG are
+// applied once per cell, to the divergence (cell_update), not once per face.
+// face_s2 takes s2 itself, for a caller that keeps it from stage to stage.
+template <int LAW, int MOB, typename V>
+__device__ __forceinline__ void face_s2(V s2, V nL, V nR, V bL, V bR, const KV<V> &k, V &phi, V &g)
+{
+    const V n2 = add_rn(nL, nR), b2 = add_rn(bL, bR);
+    const V db = sub_rn(bR, bL, k.m1), dm = sub_rn(nL, nR, k.m1);
+    V hc = k.chi;
+    if (LAW == CX_CHEMO_RECEPTOR) hc = weight(n2, k);
+    const V a = mul_rn(s2, n2);
+    if (MOB == CX_MOBILITY_CENTRAL) {
+        phi = mul_rn(mul_rn(a, b2), fma_rn(mul_rn(hc, b2), dm, db));
+    } else {
+        const V bd = donor(dm, bL, bR);
+        phi = mul_rn(a, fma_rn(mul_rn(mul_rn(hc, bd), bd), dm, mul_rn(b2, db)));
+    }
+    g = dm;
+}
 template <int LAW, int MOB, typename V>
 __device__ __forceinline__ void face(V sL, V sR, V nL, V nR, V bL, V bR, const KV<V> &k, V &phi,
                                      V &g)
 {
-    const V s2 = add_rn(sL, sR), n2 = add_rn(nL, nR), b2 = add_rn(bL, bR);
-    const V db = sub_rn(bR, bL, k.m1), dn = sub_rn(nR, nL, k.m1);
-    V hcn = k.ncChi;  // -hc
-    if (LAW == CX_CHEMO_RECEPTOR) {
-        const V q = add_rn(n2, k.two);
-        hcn = div_w(k.ncChi, mul_rn(q, q));
-    }
-    const V a = mul_rn(s2, n2);
-    if (MOB == CX_MOBILITY_CENTRAL) {
-        phi = mul_rn(mul_rn(a, b2), fma_rn(mul_rn(hcn, b2), dn, db));
-    } else {
-        const V bd = donor(dn, bL, bR);
-        phi = mul_rn(a, fma_rn(mul_rn(mul_rn(mul_rn(k.four, hcn), bd), bd), dn, mul_rn(b2, db)));
-    }
-    g = dn;
+    face_s2<LAW, MOB>(add_rn(sL, sR), nL, nR, bL, bR, k, phi, g);
 }
 
 // Four adjacent cells x0..x0+3 of one field, held as the pairs
@@ -270,6 +305,23 @@ __device__ __forceinline__ YFaces<T> row_yfaces(const Cells<T> &sL, const Cells<
     return y;
 }
 
+// The same with the face sums of sigma given.
+template <typename T, int LAW, int MOB>
+__device__ __forceinline__ YFaces<T> row_yfaces_s2(const Cells<T> &s2, const Cells<T> &nL,
+                                                   const Cells<T> &bL, const Cells<T> &nU,
+                                                   const Cells<T> &bU, const KV<P2<T>> &k)
+{
+    YFaces<T> y;
+    face_s2<LAW, MOB>(s2.E, nL.E, nU.E, bL.E, bU.E, k, y.phE, y.gE);
+    face_s2<LAW, MOB>(s2.O, nL.O, nU.O, bL.O, bU.O, k, y.phO, y.gO);
+    return y;
+}
+template <typename T>
+__device__ __forceinline__ Cells<T> y_sums(const Cells<T> &sL, const Cells<T> &sU)
+{
+    return Cells<T>{add_rn(sL.E, sU.E), add_rn(sL.O, sU.O)};
+}
+
 // x-faces of four cells: f_c lies between cells x0+c-1 and x0+c.  They are
 // computed as A = (f0, f2), B = (f1, f3) and f4; (l*, r*) are the cells
 // x0-1 and x0+4.  Faces on the walls (and past the row's end) carry zero
@@ -297,20 +349,22 @@ __device__ __forceinline__ XFaces<T> row_xfaces(const Cells<T> &s, const Cells<T
     return f;
 }
 
-// The same x-faces when every lane of the warp holds the row's next four
-// cells (the two-stage march): f4 is the right lane's f0, so each face is
-// evaluated once and no right-hand neighbour is needed.  Lane 31 takes its
-// own f0 for f4; the caller discards what depends on it.
-template <typename T, int LAW, int MOB, bool INTERIOR>
-__device__ __forceinline__ XFaces<T> row_xfaces_shfl(const Cells<T> &s, const Cells<T> &n,
-                                                     const Cells<T> &b, T ls, T ln, T lb,
-                                                     const KV<P2<T>> &k, int x0, int nx)
+// The same x-faces when the lanes hold the row's cells four by four (the
+// two-stage march, the register tiles): f4 is the right lane's f0, so each
+// face is evaluated once and no right-hand neighbour is needed.  A row lies in
+// WIDTH consecutive lanes; the last of them takes its own f0 for f4, and the
+// caller discards what depends on it.  s2: the face sums of sigma, (f0, f2)
+// and (f1, f3).
+template <typename T, int LAW, int MOB, bool INTERIOR, int WIDTH>
+__device__ __forceinline__ XFaces<T> row_xfaces_s2(const Cells<T> &s2, const Cells<T> &n,
+                                                   const Cells<T> &b, T ln, T lb,
+                                                   const KV<P2<T>> &k, int x0, int nx)
 {
     XFaces<T> f;
-    face<LAW, MOB>(pair(ls, s.O.x), s.E, pair(ln, n.O.x), n.E, pair(lb, b.O.x), b.E, k, f.phA, f.gA);
-    face<LAW, MOB>(s.E, s.O, n.E, n.O, b.E, b.O, k, f.phB, f.gB);
-    f.ph4 = __shfl_down_sync(kFull, f.phA.x, 1);
-    f.g4 = __shfl_down_sync(kFull, f.gA.x, 1);
+    face_s2<LAW, MOB>(s2.E, pair(ln, n.O.x), n.E, pair(lb, b.O.x), b.E, k, f.phA, f.gA);
+    face_s2<LAW, MOB>(s2.O, n.E, n.O, b.E, b.O, k, f.phB, f.gB);
+    f.ph4 = __shfl_down_sync(kFull, f.phA.x, 1, WIDTH);
+    f.g4 = __shfl_down_sync(kFull, f.gA.x, 1, WIDTH);
     if (!INTERIOR) {
         if (x0 == 0) f.phA.x = f.gA.x = T(0);           // west wall
         if (x0 + 1 >= nx) f.phB.x = f.gB.x = T(0);      // east wall and padding
@@ -320,10 +374,21 @@ __device__ __forceinline__ XFaces<T> row_xfaces_shfl(const Cells<T> &s, const Ce
     }
     return f;
 }
+template <typename T> __device__ __forceinline__ Cells<T> x_sums(const Cells<T> &s, T ls)
+{
+    return Cells<T>{add_rn(pair(ls, s.O.x), s.E), add_rn(s.E, s.O)};
+}
+template <typename T, int LAW, int MOB, bool INTERIOR, int WIDTH = 32>
+__device__ __forceinline__ XFaces<T> row_xfaces_shfl(const Cells<T> &s, const Cells<T> &n,
+                                                     const Cells<T> &b, T ls, T ln, T lb,
+                                                     const KV<P2<T>> &k, int x0, int nx)
+{
+    return row_xfaces_s2<T, LAW, MOB, INTERIOR, WIDTH>(x_sums(s, ls), n, b, ln, lb, k, x0, nx);
+}
 
 // u + reaction + div for one pair of cells: faces west/east and, in march
 // order, behind/ahead (DIR +1: ahead is north):
-//   b' = b + cR n b + cA div(phi),   n' = n - cN n b + cG div(g).
+//   b' = b + cR n b + cA div(phi),   n' = n - cN n b - cG div(g).
 template <typename T, int DIR>
 __device__ __forceinline__ void cell_update(P2<T> b, P2<T> n, P2<T> phW, P2<T> gW, P2<T> phE,
                                             P2<T> gE, P2<T> phB, P2<T> gB, P2<T> phA, P2<T> gA,
@@ -335,7 +400,7 @@ __device__ __forceinline__ void cell_update(P2<T> b, P2<T> n, P2<T> phW, P2<T> g
     const P2<T> divb = add_rn(sub_rn(phE, phW, k.m1), sub_rn(phN, phS, k.m1));
     const P2<T> divn = add_rn(sub_rn(gE, gW, k.m1), sub_rn(gN, gS, k.m1));
     ob = fma_rn(k.cA, divb, fma_rn(k.cR, r, b));
-    on = fma_rn(k.cG, divn, fma_rn(k.ncN, r, n));
+    on = fma_rn(k.ncG, divn, fma_rn(k.ncN, r, n));
 }
 // the four cells: even cells lie between A (west) and B (east), odd cells
 // between B and (f2, f4)
@@ -460,7 +525,7 @@ __device__ __forceinline__ void prefetch_row(const Ptrs<T> &P, long long off)
 
 template <typename T> struct Row {
     Cells<T> b, n, s;
-    T hb, hn, hs;     // lane 0: cell x0-1; lane 31: cell x0+4
+    T hb, hn, hs;     // lane 0: cell x0-1; lane 31: cell x0+4 (FP32)
     Cells<T> ub, un;  // STAGE 1: the state at the start of the step
 };
 
@@ -471,7 +536,12 @@ template <typename T> struct Row {
 // Face values do not depend on DIR (a face is always evaluated with L the
 // lower row), so both directions give bit-identical results.  CG: read
 // through L2 only (a persistent launch whose blocks read what other blocks
-// wrote earlier in the same launch).  INTERIOR: the caller guarantees that
+// wrote earlier in the same launch).  A lane's fifth x-face is the right
+// lane's first.  In FP32 every lane evaluates it again (the pass is bound by
+// HBM).  In FP64 it comes by shuffle, and the warp's last lane takes it from
+// faces that the warp evaluates once per 32 rows, each lane one row's: the
+// FP64 pipe, which bounds the pass, spends as much on an instruction with one
+// active lane as with 32.  INTERIOR: the caller guarantees that
 // every thread's cells and both x-neighbours of the warp lie inside the grid
 // (0 < x0 and x0 + 4 < nx for all threads), so the x-wall tests drop out.
 template <typename T, int LAW, int MOB, int NOISE, int STAGE, int DIR, bool CG = false,
@@ -485,7 +555,8 @@ __device__ __forceinline__ void march(const Ptrs<T> &P, int nx, int ny, long lon
     // shuffles) but load an in-row vector and store nothing
     const long long xv = INTERIOR ? (long long)x0 : min((long long)x0, pitch - kCells);
     const bool halo_l = (lane == 0) && (INTERIOR || ((x0 > 0) && (x0 < nx)));
-    const bool halo_r = (lane == 31) && (INTERIOR || (x0 + kCells < nx));
+    constexpr bool kRightOnce = sizeof(T) == 8;
+    const bool halo_r = !kRightOnce && (lane == 31) && (INTERIOR || (x0 + kCells < nx));
     const bool halo = halo_l || halo_r;
     const long long xh = halo_l ? (long long)x0 - 1 : (long long)x0 + kCells;
 
@@ -495,7 +566,7 @@ __device__ __forceinline__ void march(const Ptrs<T> &P, int nx, int ny, long lon
         else Vec<T>::load(p, v);
         return split4(v);
     };
-    auto sload = [](const T *p) -> T { return CG ? __ldcg(p) : *p; };
+    auto sload = [](const T *p) -> T { return CG ? __ldcg(p) : Vec<T>::load1(p); };
     auto load_row = [&](int r, Row<T> &R, bool own) {
         const long long off = (long long)r * pitch;
         R.b = vload(P.b + off + xv);
@@ -526,6 +597,27 @@ __device__ __forceinline__ void march(const Ptrs<T> &P, int nx, int ny, long lon
             if (CG) Vec<T>::load_cg(P.nu + off + xv, v);
             else Vec<T>::load(P.nu + off + xv, v);
             R.un = split4(v);
+        }
+    };
+    // the face right of the warp's last column in the row `it + lane` rows
+    // after the tile's first, in march order
+    T phR = T(0), gR = T(0);
+    auto right_faces = [&](int jfirst, int it, int rows) {
+        const int xe = x0 + (32 - lane) * kCells;
+        phR = gR = T(0);
+        if (it + lane < rows && (INTERIOR || xe < nx)) {
+            const int j = jfirst + DIR * (it + lane);
+            const long long off = (long long)j * pitch + xe;
+            T sL, sR;
+            if (NOISE == 0) {
+                sL = sload(P.s + off - 1);
+                sR = sload(P.s + off);
+            } else {
+                sL = nz.at((long long)j * nx + xe - 1);
+                sR = nz.at((long long)j * nx + xe);
+            }
+            face<LAW, MOB>(sL, sR, sload(P.n + off - 1), sload(P.n + off), sload(P.b + off - 1),
+                           sload(P.b + off), scalar_kv<T>(k), phR, gR);
         }
     };
     // y-faces between a lower row lo and an upper row hi
@@ -565,13 +657,21 @@ __device__ __forceinline__ void march(const Ptrs<T> &P, int nx, int ny, long lon
         T lb = __shfl_up_sync(kFull, cur.b.O.y, 1);
         T ln = __shfl_up_sync(kFull, cur.n.O.y, 1);
         T ls = __shfl_up_sync(kFull, cur.s.O.y, 1);
-        T rb = __shfl_down_sync(kFull, cur.b.E.x, 1);
-        T rn = __shfl_down_sync(kFull, cur.n.E.x, 1);
-        T rs = __shfl_down_sync(kFull, cur.s.E.x, 1);
         if (lane == 0) { lb = cur.hb; ln = cur.hn; ls = cur.hs; }
-        if (lane == 31) { rb = cur.hb; rn = cur.hn; rs = cur.hs; }
-        const XFaces<T> xf =
-            row_xfaces<T, LAW, MOB, INTERIOR>(cur.s, cur.n, cur.b, ls, ln, lb, rs, rn, rb, k, x0, nx);
+        XFaces<T> xf;
+        if (kRightOnce) {
+            if ((it & 31) == 0) right_faces(jfirst, it, rows);
+            xf = row_xfaces_shfl<T, LAW, MOB, INTERIOR>(cur.s, cur.n, cur.b, ls, ln, lb, k, x0, nx);
+            const T ph = __shfl_sync(kFull, phR, it & 31), g = __shfl_sync(kFull, gR, it & 31);
+            if (lane == 31) { xf.ph4 = ph; xf.g4 = g; }
+        } else {
+            T rb = __shfl_down_sync(kFull, cur.b.E.x, 1);
+            T rn = __shfl_down_sync(kFull, cur.n.E.x, 1);
+            T rs = __shfl_down_sync(kFull, cur.s.E.x, 1);
+            if (lane == 31) { rb = cur.hb; rn = cur.hn; rs = cur.hs; }
+            xf = row_xfaces<T, LAW, MOB, INTERIOR>(cur.s, cur.n, cur.b, ls, ln, lb, rs, rn, rb, k, x0,
+                                                   nx);
+        }
 
         // y-faces with the row ahead (a wall past the grid's first/last row)
         YFaces<T> yA;

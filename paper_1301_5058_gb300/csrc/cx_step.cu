@@ -35,22 +35,23 @@ using namespace stencil;
 // Resident blocks per SM the register budget is sized for.  FP32 Euler with
 // a static sigma field is bound by HBM bandwidth and needs every warp it can
 // get: 64 registers, 8 blocks (32 warps).  Other FP32 forms: 4 (128
-// registers); FP64 (bound by the FP64 pipe): 2.
+// registers); FP64 (bound by the FP64 pipe): 8 one-warp blocks.
 template <typename T, int NOISE, int STAGE> constexpr int step_min_blocks()
 {
-    return sizeof(T) == 4 ? ((NOISE == 0 && STAGE == 0) ? 8 : 4) : 2;
+    return sizeof(T) == 4 ? ((NOISE == 0 && STAGE == 0) ? 8 : 4) : 8;
 }
 
 template <typename T, int LAW, int MOB, int NOISE, int STAGE>
-__global__ void __launch_bounds__(kThreads, step_min_blocks<T, NOISE, STAGE>())
+__global__ void __launch_bounds__(step_threads<T>(), step_min_blocks<T, NOISE, STAGE>())
     step_kernel(Ptrs<T> P, int nx, int ny, long long pitch, KV<P2<T>> k, NoiseT<T> nz, int rows)
 {
     pass_wait();
-    const int x0 = (blockIdx.x * kThreads + threadIdx.x) * kCells;
+    constexpr int kBlockCols = step_threads<T>() * kCells;
+    const int x0 = blockIdx.x * kBlockCols + threadIdx.x * kCells;
     const int j0 = blockIdx.y * rows;
     const int jend = min(j0 + rows, ny);
-    // a block whose 512 columns touch neither x-wall takes the branch-free path
-    const bool interior = blockIdx.x > 0 && (blockIdx.x + 1) * kThreads * kCells < nx;
+    // a block whose columns touch neither x-wall takes the branch-free path
+    const bool interior = blockIdx.x > 0 && (blockIdx.x + 1) * kBlockCols < nx;
     if (blockIdx.y & 1) {
         if (interior)
             march<T, LAW, MOB, NOISE, STAGE, -1, false, true>(P, nx, ny, pitch, k, nz, x0, j0, jend);
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(kThreads, step_min_blocks<T, NOISE, STAGE>())
 template <typename T, int LAW, int MOB, int NOISE, int STAGE>
 cudaError_t launch_t(const StepArgs &a, cudaStream_t st)
 {
-    const KV<P2<T>> k = make_kv(CoefT<T>{(T)a.k.cA, (T)a.k.cChi, (T)a.k.cG, (T)a.k.cR, (T)a.k.cN});
+    const KV<P2<T>> k = make_kv(coef_t<T>(a.k));
     NoiseT<T> nz;
     nz.seed = a.sg.seed;
     nz.step = (uint64_t)a.step;
@@ -77,9 +78,9 @@ cudaError_t launch_t(const StepArgs &a, cudaStream_t st)
     set_noise_keys(nz);
     Ptrs<T> P{(const T *)a.b, (const T *)a.n, (const T *)a.s, (const T *)a.bu,
               (const T *)a.nu, (T *)a.bo, (T *)a.no};
-    const dim3 grid((a.nx + kThreads * kCells - 1) / (kThreads * kCells),
-                    (a.ny + a.rows - 1) / a.rows);
-    return launch_pass(step_kernel<T, LAW, MOB, NOISE, STAGE>, grid, kThreads, 0, st, P, a.nx, a.ny,
+    constexpr int cols = step_threads<T>() * kCells;
+    const dim3 grid((a.nx + cols - 1) / cols, (a.ny + a.rows - 1) / a.rows);
+    return launch_pass(step_kernel<T, LAW, MOB, NOISE, STAGE>, grid, step_threads<T>(), 0, st, P, a.nx, a.ny,
                        a.pitch, k, nz, a.rows);
 }
 
