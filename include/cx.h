@@ -248,7 +248,11 @@ int cx_set_step(cx_ctx *c, int64_t step);
  * small grids so that about four tiles per SM are launched (sixteen
  * one-warp tiles with two stages and static sigma, eight four-warp tiles
  * with sigma redrawn per step); cx_get_tile_rows reports the height in
- * effect. */
+ * effect.  While neither a height nor a depth (cx_set_time_block) has been
+ * set, cx_step takes several time steps per pass where that is faster and the
+ * result the same bits: an FP32 grid of up to about 2500^2 cells (4000^2 with
+ * sigma redrawn per step) on tiles that blocks hold in registers, an FP64 strip
+ * (ny = 1, static sigma) on one-warp tiles. */
 int cx_set_tile_rows(cx_ctx *c, int32_t rows);
 int cx_get_tile_rows(cx_ctx *c, int32_t *rows);
 
@@ -301,7 +305,10 @@ int cx_batch_set_stream(cx_batch *b, void *stream);
 /* Performance knobs, none of which changes any result bit:
  *   tile_rows   rows per tile of the step kernel (1..4096; the tiles of
  *               both depths; default 128 for FP32 batches, which take two
- *               stages per pass, 32 for FP64 ones);
+ *               stages per pass, 32 for FP64 ones).  A batch whose knobs and
+ *               depth were never set chooses for itself, as a single grid
+ *               does: fewer rows where it would leave the GPU idle, or
+ *               several steps per pass on register tiles;
  *   graph_steps steps captured per CUDA graph and replayed (0: plain
  *               launches; rounded up to even for Euler; default 64);
  *   group_bytes if > 0, instances are cut into consecutive groups whose

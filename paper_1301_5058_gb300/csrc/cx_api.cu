@@ -262,6 +262,19 @@ cx::Coef cx::make_coef(const cx_grid &g, const cx_params &p, double dt)
     return k;
 }
 
+// The modelled time per step (us) of the row marches on `cells` cells of an
+// FP32 state, fitted to measured single grids: Euler, static sigma 3.1 (512^2),
+// 10.1 (2048^2), 32.4 (4096^2); Euler, per-step sigma 13.1 (1024^2), 59
+// (4096^2); Heun 8.9 (1024^2), 21.0 (2048^2); Heun, per-step sigma 19.1
+// (1024^2), 37.1 (2048^2), 89 (4096^2).  The register tiles take 1.2, 9.0 and
+// 33; 4.6 and 53; 6.3 and 20.0; 8.3, 25.0 and 93 there, so the line lies near
+// 2500^2 for a static sigma and near 4000^2 for one drawn every step.
+double cx::march_us(double cells, bool heun, bool per_step)
+{
+    if (heun) return per_step ? 10.0 + 4.6e-6 * cells : 4.6 + 3.7e-6 * cells;
+    return per_step ? 10.0 + 2.9e-6 * cells : 2.3 + 1.85e-6 * cells;
+}
+
 extern "C" {
 
 int cx_version(void) { return CX_VERSION; }
@@ -437,6 +450,30 @@ int cx_set_stream(cx_ctx *c, void *stream)
     return CX_OK;
 }
 
+// Whether a call of n_steps steps takes several steps per pass: on register
+// tiles (FP32) or strips (FP64, one row, static sigma), where depth and tile
+// height were left to the library and the modelled tiles are faster than the
+// marches.
+static bool use_tiles(cx_ctx *c, int64_t n_steps)
+{
+    if (c->tile_rows > 0 || c->depth_set || n_steps < 1) return false;
+    if (c->plan_for != n_steps) {
+        const bool heun = c->p.scheme == CX_SCHEME_HEUN;
+        const bool per_step = c->p.noise_mode == CX_NOISE_PER_STEP;
+        const cx::TileGrid g{c->g.nx, c->g.ny, 1};
+        double us = HUGE_VAL, march = 0.0;
+        if (c->prec == CX_PREC_F32) {
+            us = cx::plan_tiles(&g, 1, c->num_sms, heun, per_step, n_steps, &c->plan);
+            march = cx::march_us((double)c->g.nx * c->g.ny, heun, per_step);
+        } else if (c->g.ny == 1 && !per_step) {
+            us = cx::plan_strips(&g, 1, c->num_sms, c->p.chemo_law, heun, n_steps, &c->plan, &march);
+        }
+        c->plan_tiles = us < march;
+        c->plan_for = n_steps;
+    }
+    return c->plan_tiles != 0;
+}
+
 int cx_step(cx_ctx *c, int64_t n_steps)
 {
     cx::NvtxRange range("cx_step");
@@ -459,7 +496,29 @@ int cx_step(cx_ctx *c, int64_t n_steps)
     a.s = c->sigma;
     const bool heun = c->p.scheme == CX_SCHEME_HEUN;
     int64_t m = 0;
-    if (c->time_block == 2) {
+    if (use_tiles(c, n_steps)) {
+        // as few passes as the plan allows, of equal length
+        cx::TilePlan p = c->plan;
+        const int64_t passes = (n_steps + p.steps - 1) / p.steps;
+        for (int64_t i = 0; i < passes; ++i) {
+            p.steps = (int)((n_steps - m + passes - i - 1) / (passes - i));
+            a.b = c->b[c->cur];
+            a.n = c->n[c->cur];
+            a.bo = c->b[c->cur ^ 1];
+            a.no = c->n[c->cur ^ 1];
+            a.step = c->step;
+            cx::TileLaunch t{};
+            t.grid = &a;
+            const cudaError_t e =
+                c->prec == CX_PREC_F64
+                    ? cx::launch_strip(a.law, a.mob, t, p, c->stream)
+                    : cx::launch_tile(a.law, a.mob, a.sg.per_step != 0, t, p, c->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "tile kernel launch");
+            c->cur ^= 1;
+            c->step += p.steps;
+            m += p.steps;
+        }
+    } else if (c->time_block == 2) {
         // two stages per pass: two Euler steps, or one whole Heun step
         const int64_t per_pass = heun ? 1 : 2;
         for (; m + per_pass <= n_steps; m += per_pass) {
@@ -824,6 +883,7 @@ int cx_set_time_block(cx_ctx *c, int32_t stages)
     if (stages != 1 && stages != 2)
         return fail(CX_ERR_INVALID_ARG, "time block %d: must be 1 or 2 stages per pass", stages);
     c->time_block = stages;
+    c->depth_set = 1;
     return CX_OK;
 }
 

@@ -5,7 +5,10 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
+#include <map>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "cx_internal.h"
@@ -34,6 +37,13 @@ constexpr int kDiagBlocksPerInst = 64;
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Register tiles (cx_tile.cu) of every instance for passes of plan.steps steps.
+struct TileWork {
+    cx::TilePlan plan;
+    int4 *d = nullptr;
+    std::vector<int> begin;  // first tile of each instance (+ total)
+};
+
 }  // namespace
 
 struct cx_batch {
@@ -55,7 +65,15 @@ struct cx_batch {
     std::vector<int> work_begin;  // first work item of each instance (+ total)
     int4 *d_work2 = nullptr;      // 120-column tiles (two stages per pass)
     std::vector<int> work2_begin;
-    int rows = 32;
+    int rows = 32;                  // tile height set, or reported as the default
+    int march_rows = 32;            // tile height in effect
+    bool tuned = false;             // heights or depth were set: the marches run as told
+    int num_sms = 1;
+    std::vector<cx::TileGrid> sizes;  // the instances' distinct sizes
+    int64_t plan_for = 0;           // steps that `plan` was made for (0: none yet)
+    bool tiles = false;             // passes run on register tiles
+    cx::TilePlan plan{};
+    std::vector<TileWork> tile_work;  // by pass length
     int graph_steps = 64;
     long long group_bytes = 0;
     int time_block = 1;             // explicit stages per pass (1 or 2)
@@ -93,6 +111,8 @@ void free_batch(cx_batch *B)
     if (B->d_inst) cudaFree(B->d_inst);
     if (B->d_work) cudaFree(B->d_work);
     if (B->d_work2) cudaFree(B->d_work2);
+    for (TileWork &t : B->tile_work)
+        if (t.d) cudaFree(t.d);
     if (B->d_part) cudaFree(B->d_part);
     if (B->d_res) cudaFree(B->d_res);
     if (B->h_res) cudaFreeHost(B->h_res);
@@ -116,7 +136,7 @@ int build_work(cx_batch *B)
         for (int i = 0; i < B->count; ++i) {
             begin[i] = (int)w.size();
             const int tx = (B->g[i].nx + cols - 1) / cols;
-            const int ty = (B->g[i].ny + B->rows - 1) / B->rows;
+            const int ty = (B->g[i].ny + B->march_rows - 1) / B->march_rows;
             for (int y = 0; y < ty; ++y)
                 for (int x = 0; x < tx; ++x) w.push_back(make_int4(i, x, y, 0));
         }
@@ -126,6 +146,111 @@ int build_work(cx_batch *B)
         BX_CUDA(cudaMalloc((void **)&d, w.size() * sizeof(int4)), "work list allocation");
         BX_CUDA(cudaMemcpy(d, w.data(), w.size() * sizeof(int4), cudaMemcpyHostToDevice),
                 "work list upload");
+    }
+    return CX_OK;
+}
+
+// Tile height of a batch that has not been tuned: the default (B->rows), or
+// fewer rows so that a small batch fills the GPU: in FP32 sixteen one-warp
+// tiles of the two-stage march per SM; in FP64 the height r with the least
+// ceil(tiles / FP64 units) (r + 1/2), as for a single grid.
+int auto_rows(const cx_batch *B)
+{
+    const bool f64 = B->prec == CX_PREC_F64;
+    const long long cols = f64 ? tile_cols(B->prec) : kFusedTileCols, units = 4LL * B->num_sms;
+    long long columns = 0;  // tile columns x rows of all instances
+    for (const cx_grid &g : B->g) columns += (g.nx + cols - 1) / cols * g.ny;
+    if (!f64) {
+        const long long r = columns / (4 * units);
+        return (int)(r < 8 ? 8 : r < B->rows ? r : B->rows);
+    }
+    long long best = 1;
+    double cost = 0.0;
+    for (long long r = 1; r <= B->rows; ++r) {
+        long long tiles = 0;
+        for (const cx::TileGrid &s : B->sizes)
+            tiles += (s.nx + cols - 1) / cols * ((s.ny + r - 1) / r) * s.count;
+        const double now = (double)((tiles + units - 1) / units) * ((double)r + 0.5);
+        if (cost == 0.0 || now <= cost) {
+            cost = now;
+            best = r;
+        }
+    }
+    return (int)best;
+}
+
+// Whether runs of `steps` steps take several steps per pass, as a single grid
+// does: an untuned batch on register tiles (FP32) or strips (FP64, every
+// instance one row high, static sigma), where they are modelled to be faster.
+bool use_tiles(cx_batch *B, int64_t steps)
+{
+    if (B->tuned) return false;
+    if (B->plan_for != steps) {
+        const bool heun = B->scheme == CX_SCHEME_HEUN, per_step = B->noise != 0;
+        const cx::TileGrid *sizes = B->sizes.data();
+        const int ns = (int)B->sizes.size();
+        double us = HUGE_VAL, march = 0.0;
+        if (B->prec == CX_PREC_F32) {
+            us = cx::plan_tiles(sizes, ns, B->num_sms, heun, per_step, steps, &B->plan);
+            double cells = 0.0;  // computed by the march, halo rows and idle columns included
+            for (const cx::TileGrid &s : B->sizes)
+                cells += (double)s.count * ((s.nx + kFusedTileCols - 1) / kFusedTileCols * kFusedTileCols) *
+                         s.ny * (B->march_rows + 2) / B->march_rows;
+            march = cx::march_us(cells, heun, per_step);
+        } else if (!per_step && std::all_of(B->sizes.begin(), B->sizes.end(),
+                                            [](const cx::TileGrid &s) { return s.ny == 1; })) {
+            us = cx::plan_strips(sizes, ns, B->num_sms, B->law, heun, steps, &B->plan, &march);
+        }
+        B->tiles = us < march;
+        B->plan_for = steps;
+    }
+    return B->tiles;
+}
+
+// Steps of the next register-tile pass of `left`: as few passes as the plan
+// allows, of equal length.
+int tile_pass_steps(const cx_batch *B, int64_t left)
+{
+    const int64_t passes = (left + B->plan.steps - 1) / B->plan.steps;
+    return (int)((left + passes - 1) / passes);
+}
+
+// The tiles for passes of the plan's shape and `steps` steps, built once.
+TileWork *find_tiles(cx_batch *B, int steps)
+{
+    for (TileWork &t : B->tile_work)
+        if (t.plan.steps == steps && t.plan.lx == B->plan.lx && t.plan.r == B->plan.r &&
+            t.plan.threads == B->plan.threads)
+            return &t;
+    return nullptr;
+}
+
+// Builds what the passes of a run of `left` steps need (not during a capture).
+int build_tiles(cx_batch *B, int64_t left)
+{
+    while (left > 0) {
+        const int steps = tile_pass_steps(B, left);
+        left -= steps;
+        if (find_tiles(B, steps)) continue;
+        TileWork t;
+        t.plan = B->plan;
+        t.plan.steps = steps;
+        std::vector<int4> w;
+        t.begin.assign(B->count + 1, 0);
+        for (int i = 0; i < B->count; ++i) {
+            t.begin[i] = (int)w.size();
+            const int tx = cx::tiles_x(B->g[i].nx, t.plan), ty = cx::tiles_y(B->g[i].ny, t.plan);
+            for (int y = 0; y < ty; ++y)
+                for (int x = 0; x < tx; ++x) w.push_back(make_int4(i, x, y, 0));
+        }
+        t.begin[B->count] = (int)w.size();
+        BX_CUDA(cudaMalloc((void **)&t.d, w.size() * sizeof(int4)), "tile list allocation");
+        const cudaError_t e = cudaMemcpy(t.d, w.data(), w.size() * sizeof(int4), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            cudaFree(t.d);
+            return bcuda(e, "tile list upload");
+        }
+        B->tile_work.push_back(t);
     }
     return CX_OK;
 }
@@ -169,10 +294,10 @@ cudaError_t one_step(cx_batch *B, int i0, int i1, int parity, int step_off)
     const int4 *work = B->d_work + w0;
     const cx::BatchNoise nz = pass_noise(B, step_off);
     cudaError_t e = cx::launch_batch_step(B->prec, B->law, B->mob, B->d_inst, work, w1 - w0,
-                                          parity, B->rows, 0, nz, B->stream);
+                                          parity, B->march_rows, 0, nz, B->stream);
     if (e == cudaSuccess && B->scheme == CX_SCHEME_HEUN)
         e = cx::launch_batch_step(B->prec, B->law, B->mob, B->d_inst, work, w1 - w0, parity,
-                                  B->rows, 1, nz, B->stream);
+                                  B->march_rows, 1, nz, B->stream);
     return e;
 }
 
@@ -186,10 +311,25 @@ cudaError_t one_pass(cx_batch *B, int i0, int i1, int *parity, int64_t left, int
                      int *steps)
 {
     const bool heun = B->scheme == CX_SCHEME_HEUN;
+    if (B->tiles) {
+        *steps = tile_pass_steps(B, left);
+        const TileWork *t = find_tiles(B, *steps);
+        if (!t) return cudaErrorInvalidValue;
+        cx::TileLaunch a{};
+        a.inst = B->d_inst;
+        a.work = t->d + t->begin[i0];
+        a.nwork = t->begin[i1] - t->begin[i0];
+        a.parity = *parity;
+        a.nz = pass_noise(B, step_off);
+        *parity ^= 1;
+        return B->prec == CX_PREC_F64
+                   ? cx::launch_strip(B->law, B->mob, a, t->plan, B->stream)
+                   : cx::launch_tile(B->law, B->mob, B->noise != 0, a, t->plan, B->stream);
+    }
     if (B->time_block == 2 && (heun || left >= 2)) {
         const int w0 = B->work2_begin[i0], w1 = B->work2_begin[i1];
         const cudaError_t e = cx::launch_batch_fused(B->prec, B->law, B->mob, B->d_inst,
-                                                     B->d_work2 + w0, w1 - w0, *parity, B->rows,
+                                                     B->d_work2 + w0, w1 - w0, *parity, B->march_rows,
                                                      heun ? 1 : 0, pass_noise(B, step_off),
                                                      B->stream);
         *parity ^= 1;
@@ -258,7 +398,7 @@ int run_resident(cx_batch *B, int i0, int i1, int par, int64_t left, int64_t ste
         BX_CUDA(cudaMemsetAsync(B->d_barrier, 0, 8, B->stream), "barrier reset");
         BX_CUDA(mark_step(B, step), "step mark");
         BX_CUDA(cx::launch_batch_resident(B->prec, B->law, B->mob, B->d_inst, B->d_work + w0, w1 - w0,
-                                          par, B->rows, chunk, B->scheme == CX_SCHEME_HEUN,
+                                          par, B->march_rows, chunk, B->scheme == CX_SCHEME_HEUN,
                                           B->d_barrier, B->spin_limit, pass_noise(B, 0), B->stream),
                 "resident batch launch");
         step += chunk;
@@ -364,6 +504,17 @@ int cx_batch_create(int32_t count, const cx_grid *grids, const cx_params *params
     if (e == cudaSuccess && B->noise) e = cudaMemset(B->d_step, 0, sizeof(long long));
     if (e != cudaSuccess) { cudaGetLastError(); free_batch(B); return bcuda(e, "batch tables"); }
     if (const char *s = getenv("CX_BARRIER_SPIN_LIMIT")) B->spin_limit = atoll(s);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&B->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        B->num_sms < 1) {
+        cudaGetLastError();
+        B->num_sms = 1;  // only the choice of tiles uses it
+    }
+    std::map<std::pair<int, int>, int> sizes;
+    for (int i = 0; i < count; ++i) sizes[{grids[i].nx, grids[i].ny}] += 1;
+    for (const auto &z : sizes) B->sizes.push_back(cx::TileGrid{z.first.first, z.first.second, z.second});
+    B->march_rows = auto_rows(B);
     int rc = build_work(B);
     if (rc) { free_batch(B); return rc; }
     build_groups(B);
@@ -407,8 +558,9 @@ int cx_batch_set_tuning(cx_batch *B, int32_t tile_rows, int32_t graph_steps, int
                                          "resident_steps 0..1000000");
     BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before retuning");
     drop_graphs(B);
-    const bool new_rows = tile_rows != B->rows;
-    B->rows = tile_rows;
+    const bool new_rows = tile_rows != B->march_rows;
+    B->rows = B->march_rows = tile_rows;
+    B->tuned = true;
     B->graph_steps = (B->scheme == CX_SCHEME_EULER && (graph_steps & 1)) ? graph_steps + 1 : graph_steps;
     B->group_bytes = group_bytes;
     B->resident_steps = resident_steps;
@@ -441,6 +593,7 @@ int cx_batch_set_time_block(cx_batch *B, int32_t stages)
     BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before retuning");
     drop_graphs(B);
     B->time_block = stages;
+    B->tuned = true;
     return CX_OK;
 }
 
@@ -460,6 +613,18 @@ int cx_batch_step(cx_batch *B, int64_t n_steps)
     if (rc) return rc;
     if (n_steps < 0) return bfail(CX_ERR_INVALID_ARG, "n_steps < 0");
     if (n_steps == 0) return CX_OK;
+    const bool whole = B->graph_steps > 0 && n_steps >= B->graph_steps;  // at least one graph
+    const bool was_tiles = B->tiles;
+    B->tiles = use_tiles(B, whole ? B->graph_steps : n_steps);
+    if (B->tiles != was_tiles) {
+        BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before new graphs");
+        drop_graphs(B);
+    }
+    if (B->tiles) {
+        rc = whole ? build_tiles(B, B->graph_steps) : CX_OK;
+        if (rc == CX_OK) rc = build_tiles(B, whole ? n_steps % B->graph_steps : n_steps);
+        if (rc) return rc;
+    }
     const int ngroups = (int)B->group_first.size() - 1;
     if (B->graph_steps > 0 && (int)B->gexec[0].size() != ngroups) {
         drop_graphs(B);

@@ -158,6 +158,7 @@ int validate_params(const cx_grid *g, const cx_params *p);
 int resolve_time_step(const cx_grid *g, const cx_params *p, double *dt);
 Coef make_coef(const cx_grid &g, const cx_params &p, double dt);
 double envelope_level(const cx_params &p);
+double march_us(double cells, bool heun, bool per_step);
 
 // Batched stepping and diagnostics (cx_batch.cu).  `inst` is the device
 // instance table, `work` the device work list (int4: instance, tile x,
@@ -195,6 +196,49 @@ cudaError_t launch_batch_resident(int prec, int law, int mob, const void *inst, 
                                   void *barrier, long long spin_limit, const BatchNoise &nz,
                                   cudaStream_t st);
 
+// A pass of the register-tile kernel (cx_tile.cu; FP32): `steps` time steps on
+// tiles of 4 lx columns and (threads / lx) r rows that overlap by the halo
+// that the pass's stages need.
+struct TilePlan {
+    int steps, lx, r, threads;
+    bool heun;
+    int stages() const { return heun ? 2 * steps : steps; }
+    int width() const { return 4 * lx; }
+    int height() const { return threads / lx * r; }
+    int halo_x() const { return (stages() + 3) / 4 * 4; }  // whole groups of four cells
+    int halo_y() const { return stages(); }
+};
+// Tiles along a side of n cells; the first and the last lie against the walls
+// and need no halo there.
+inline int tile_count(int n, int size, int halo)
+{
+    const int step = size - 2 * halo;
+    return n <= size ? 1 : 1 + (n - size + step - 1) / step;
+}
+inline int tiles_x(int nx, const TilePlan &p) { return tile_count(nx, p.width(), p.halo_x()); }
+inline int tiles_y(int ny, const TilePlan &p) { return tile_count(ny, p.height(), p.halo_y()); }
+struct TileGrid {
+    int nx, ny, count;  // `count` grids of this size
+};
+double plan_tiles(const TileGrid *grids, int count, int sms, bool heun, bool per_step,
+                  long long steps, TilePlan *best);
+// What a pass runs on: one grid (law, mobility and stage of the arguments not
+// used), or a batch's work list of (instance, tile x, tile y).
+struct TileLaunch {
+    const StepArgs *grid;
+    const void *inst;
+    const int4 *work;
+    int nwork, parity;
+    BatchNoise nz;
+};
+cudaError_t launch_tile(int law, int mob, bool per_step, const TileLaunch &a, const TilePlan &p,
+                        cudaStream_t st);
+// The same for FP64 strips with a static sigma (cx_strip.cu); *march: the
+// march's modelled time per step.
+double plan_strips(const TileGrid *grids, int count, int sms, int law, bool heun, long long steps,
+                   TilePlan *best, double *march);
+cudaError_t launch_strip(int law, int mob, const TileLaunch &a, const TilePlan &p, cudaStream_t st);
+
 }  // namespace cx
 
 struct cx_ctx {
@@ -215,6 +259,10 @@ struct cx_ctx {
     int num_sms;          // streaming multiprocessors of that device
     int tile_rows;        // rows per step-kernel tile (0: automatic)
     int time_block;       // explicit stages per pass over the grid (1 or 2)
+    int depth_set;        // time_block was chosen by cx_set_time_block
+    int64_t plan_for;     // cx_step's n_steps that `plan` was made for (0: none yet)
+    int plan_tiles;       // that call runs on register tiles
+    cx::TilePlan plan;
     cx::DiagScratch diag;
     double *h_diag;       // pinned [8]
     // staged uploads (cx_stage_state / cx_commit_state), created on first use
