@@ -132,7 +132,6 @@ void free_buffers(cx_ctx *c)
     c->copy_stream = nullptr;
     c->staged = c->stage_free = nullptr;
     if (c->diag.partials) cudaFree(c->diag.partials);
-    if (c->diag.result) cudaFree(c->diag.result);
     if (c->h_diag) cudaFreeHost(c->h_diag);
     c->sigma = nullptr;
     c->diag.partials = c->diag.result = nullptr;
@@ -192,8 +191,8 @@ int alloc_ctx(const cx_grid *g, const cx_params *p, uint64_t seed, double dt, cx
     }
     c->diag.blocks = cx::diag_blocks_for(g->ny);
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->diag.partials, 8 * sizeof(double) * c->diag.blocks);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->diag.result, 8 * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_diag, 8 * sizeof(double));
+    c->diag.result = c->h_diag;  // the last kernel writes the record to the host itself
     for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
         e = cudaMemset(c->b[q], 0, bytes);
         if (e == cudaSuccess) e = cudaMemset(c->n[q], 0, bytes);
@@ -583,9 +582,6 @@ int cx_diagnostics(cx_ctx *c, cx_diag *out)
     CX_CUDA(cx::launch_diagnostics(c->prec, c->b[c->cur], c->n[c->cur], c->g.nx, c->g.ny,
                                    c->pitch, bth, c->diag, c->stream),
             "diagnostics launch");
-    CX_CUDA(cudaMemcpyAsync(c->h_diag, c->diag.result, 8 * sizeof(double), cudaMemcpyDeviceToHost,
-                            c->stream),
-            "diagnostics copy");
     CX_CUDA(cudaStreamSynchronize(c->stream), "diagnostics synchronize");
     const double *h = c->h_diag;
     const double area = c->g.dx * c->g.dx;
@@ -644,8 +640,14 @@ int cx_get_field(cx_ctx *c, int32_t which, void *host, int32_t dtype, size_t cou
     // with per-step noise, sigma is the field the next step will use
     if (which == CX_FIELD_SIGMA && c->p.noise_mode == CX_NOISE_PER_STEP)
         CX_CUDA(fill_sigma(c, c->step), "sigma regeneration");
-    // the array in natural in-row order for the copy, and back afterwards
     void *f = field_ptr(c, which);
+    if (void *view = cx::pinned_view(host, count * (dtype == CX_F64 ? 8 : 4))) {
+        CX_CUDA(cx::launch_read_field(c->prec, f, c->g.nx, c->g.ny, c->pitch, view, dtype, c->stream),
+                "field read");
+        CX_CUDA(cudaStreamSynchronize(c->stream), "field read synchronize");
+        return CX_OK;
+    }
+    // the array in natural in-row order for the copy, and back afterwards
     CX_CUDA(cx::launch_pair_order(c->prec, f, c->g.nx, c->g.ny, c->pitch, c->stream), "reorder");
     if (dtype == state_dtype) {
         CX_CUDA(copy_rows(host, row, f, (size_t)c->pitch * c->elem, row, c->g.ny,

@@ -78,8 +78,9 @@ __global__ void __launch_bounds__(reduce::kThreads)
 }
 
 __global__ void __launch_bounds__(reduce::kThreads)
-    batch_diag_final(const double *__restrict__ part, int blocks, double *__restrict__ out)
+    batch_diag_final(const double *part, int blocks, double *out)
 {
+    pass_wait();
     const int i = blockIdx.x;
     reduce::Acc a = reduce::empty_acc();
     for (int r = threadIdx.x; r < blocks; r += reduce::kThreads)
@@ -179,9 +180,8 @@ cudaError_t launch_batch_diag(int prec, const void *inst, int first, int count, 
                                                                   first, parity, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    batch_diag_final<<<count, reduce::kThreads, 0, st>>>(part + 8LL * first * blocks, blocks,
-                                                         out + 8LL * first);
-    return cudaGetLastError();
+    return launch_pass(batch_diag_final, count, reduce::kThreads, 0, st, part + 8LL * first * blocks,
+                       blocks, out + 8LL * first);
 }
 
 size_t inst_dev_bytes(int prec) { return prec == CX_PREC_F64 ? sizeof(InstDev<double>) : sizeof(InstDev<float>); }

@@ -87,7 +87,7 @@ struct cx_batch {
     int64_t step = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    double *d_part = nullptr, *d_res = nullptr, *h_res = nullptr;
+    double *d_part = nullptr, *h_res = nullptr;  // h_res: pinned, written by the diagnostics kernel
 };
 
 namespace {
@@ -114,7 +114,6 @@ void free_batch(cx_batch *B)
     for (TileWork &t : B->tile_work)
         if (t.d) cudaFree(t.d);
     if (B->d_part) cudaFree(B->d_part);
-    if (B->d_res) cudaFree(B->d_res);
     if (B->h_res) cudaFreeHost(B->h_res);
     if (B->d_barrier) cudaFree(B->d_barrier);
     if (B->d_step) cudaFree(B->d_step);
@@ -496,7 +495,6 @@ int cx_batch_create(int32_t count, const cx_grid *grids, const cx_params *params
     e = cudaMalloc(&B->d_inst, B->h_inst.size());
     if (e == cudaSuccess) e = cudaMemcpy(B->d_inst, B->h_inst.data(), B->h_inst.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc((void **)&B->d_part, 8 * sizeof(double) * (size_t)count * kDiagBlocksPerInst);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&B->d_res, 8 * sizeof(double) * (size_t)count);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&B->h_res, 8 * sizeof(double) * (size_t)count);
     if (e == cudaSuccess) e = cudaMalloc(&B->d_barrier, cx::grid_barrier_bytes());
     if (e == cudaSuccess) e = cudaMemset(B->d_barrier, 0, cx::grid_barrier_bytes());
@@ -687,11 +685,8 @@ int cx_batch_diagnostics(cx_batch *B, cx_diag *out)
     if (rc) return rc;
     if (!out) return bfail(CX_ERR_INVALID_ARG, "out must not be NULL");
     BX_CUDA(cx::launch_batch_diag(B->prec, B->d_inst, 0, B->count, kDiagBlocksPerInst, B->cur,
-                                  B->d_part, B->d_res, B->stream),
+                                  B->d_part, B->h_res, B->stream),
             "batch diagnostics launch");
-    BX_CUDA(cudaMemcpyAsync(B->h_res, B->d_res, 8 * sizeof(double) * (size_t)B->count,
-                            cudaMemcpyDeviceToHost, B->stream),
-            "batch diagnostics copy");
     BX_CUDA(cudaStreamSynchronize(B->stream), "batch diagnostics synchronize");
     rc = check_barrier(B);
     if (rc) return rc;
@@ -748,6 +743,13 @@ int cx_batch_get_field(cx_batch *B, int32_t index, int32_t which, void *host, in
     if (!host) return bfail(CX_ERR_INVALID_ARG, "host must not be NULL");
     const int sd = B->prec == CX_PREC_F64 ? CX_F64 : CX_F32;
     const size_t row = (size_t)B->g[index].nx * B->elem;
+    if (void *view = cx::pinned_view(host, count * (dtype == CX_F64 ? 8 : 4))) {
+        BX_CUDA(cx::launch_read_field(B->prec, batch_field(B, index, which), B->g[index].nx,
+                                      B->g[index].ny, B->pitch[index], view, dtype, B->stream),
+                "field read");
+        BX_CUDA(cudaStreamSynchronize(B->stream), "field read synchronize");
+        return CX_OK;
+    }
     std::vector<unsigned char> tmp;
     void *dst = host;
     if (dtype != sd) {

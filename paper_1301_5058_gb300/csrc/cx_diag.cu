@@ -45,8 +45,9 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 __global__ void __launch_bounds__(kThreads)
-    diag_final(const double *__restrict__ part, int blocks, double *__restrict__ out)
+    diag_final(const double *part, int blocks, double *out)
 {
+    pass_wait();
     Acc a = empty_acc();
     for (int r = threadIdx.x; r < blocks; r += kThreads) combine(a, load_acc(part + 8LL * r));
     a = block_reduce(a);
@@ -84,8 +85,7 @@ cudaError_t launch_diagnostics(int prec, const void *b, const void *n, int nx, i
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    diag_final<<<1, kThreads, 0, st>>>(s.partials, s.blocks, s.result);
-    return cudaGetLastError();
+    return launch_pass(diag_final, 1, kThreads, 0, st, s.partials, s.blocks, s.result);
 }
 
 }  // namespace cx

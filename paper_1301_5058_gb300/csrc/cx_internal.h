@@ -133,9 +133,17 @@ __host__ __device__ __forceinline__ long long pair_col(long long i)
 // natural in-row order and the pair order (either way).
 cudaError_t launch_pair_order(int prec, void *a, int nx, int ny, long long pitch, cudaStream_t st);
 
+// The address under which a kernel may write the `bytes` bytes at `host`, or
+// nullptr unless all of them are pinned (cx_read.cu).
+void *pinned_view(void *host, size_t bytes);
+// A field in pair order -> packed rows of nx elements in natural order and of
+// type `dtype` (CX_F64 / CX_F32) at `dst`, device or pinned host memory.
+cudaError_t launch_read_field(int prec, const void *field, int nx, int ny, long long pitch, void *dst,
+                              int dtype, cudaStream_t st);
+
 struct DiagScratch {
     double *partials;  // [blocks][8]
-    double *result;    // [8] on the device
+    double *result;    // [8], device or pinned host memory
     int blocks;
 };
 int diag_blocks_for(int ny);
