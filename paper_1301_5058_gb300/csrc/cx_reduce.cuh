@@ -23,13 +23,23 @@ struct Acc {
     long long cnt;  // cells with b >= threshold
 };
 
+// a < b for numbers that are not NaN (an accumulator never is), compared as
+// integers: a double comparison holds a scheduler's FP64 unit for 64 cycles per
+// warp, and three of the five FP64 operations of a fold were comparisons
+// (diagnostics of 1024^2 in FP32 40.5 -> 28.6 us, 256^2 23.0 -> 17.3).
+__device__ __forceinline__ bool less(double a, double b)
+{
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return (x ^ ((x >> 63) & 0x7fffffffffffffffLL)) < (y ^ ((y >> 63) & 0x7fffffffffffffffLL));
+}
+
 __device__ __forceinline__ void combine(Acc &a, const Acc &o)
 {
     a.sb += o.sb;
     a.sn += o.sn;
-    a.mnb = fmin(a.mnb, o.mnb);
-    a.mnn = fmin(a.mnn, o.mnn);
-    a.mxb = fmax(a.mxb, o.mxb);
+    if (less(o.mnb, a.mnb)) a.mnb = o.mnb;
+    if (less(o.mnn, a.mnn)) a.mnn = o.mnn;
+    if (less(a.mxb, o.mxb)) a.mxb = o.mxb;
     a.r2 = max(a.r2, o.r2);
     a.bad |= o.bad;
     a.cnt += o.cnt;
@@ -69,7 +79,7 @@ __device__ __forceinline__ Acc block_reduce(Acc a)
     __syncthreads();
     if (w == 0) {
         a = lane < kThreads / 32 ? warp_acc[lane] : empty_acc();
-        for (int d = 16; d > 0; d >>= 1) combine(a, shfl_down(a, d));
+        for (int d = kThreads / 64; d > 0; d >>= 1) combine(a, shfl_down(a, d));
     }
     return a;
 }
