@@ -26,16 +26,25 @@
 // Members share no data, so member e of an E-member network computes what a
 // one-member network computes, bit for bit.
 //
-// Tensor-core tiles.  A CTA of 128 threads computes D (128 x 256, FP32) =
-// A (128 x K) B (256 x K)^T: A and B are staged K-major in shared memory,
-// 128 columns of K at a time, in the no-swizzle canonical layout (8 x 8
+// Tensor-core tiles.  A CTA of 512 threads computes D (128 x 64, FP32) =
+// A (128 x K) B (64 x K)^T: A and B are staged K-major in shared memory, up to
+// 256 columns of K at a time, in the no-swizzle canonical layout (8 x 8
 // core matrices of 128 contiguous bytes); one elected thread issues
-// tcgen05.mma (M = 128, N = 256, K = 16 each) into 256 columns of tensor
+// tcgen05.mma (M = 128, N = 64, K = 16 each) into 64 columns of tensor
 // memory and commits them to an mbarrier; every thread waits on it (a
 // bounded wait) and reads its row (TMEM lane = tile row) with tcgen05.ld.
 // The operands are small and L2-resident (at most 256 x 8192 bf16 per
 // member), and the forward's A operand is computed, not copied, so the
 // staging is plain 16-byte loads rather than TMA.
+//
+// What bounds a training step is the latency of a handful of tiles (8 members
+// x 256 rows), most of it tanhf and operand staging, so the 256 hidden columns
+// are cut into four tiles of 64: four times as many CTAs, each with a quarter
+// of the epilogue.  In the forward pass the four form a cluster: each computes
+// a quarter of H1 and writes it into the A operand of all four (distributed
+// shared memory), and the four partial sums of Y meet in the same way.  With
+// the launches overlapped (launch_pass), a training step of 8 members x 256
+// rows takes 38 us; one CTA per 128 x 256 tile took 89.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>
@@ -65,26 +74,26 @@ static_assert(NPARAM == CX_MLP_PARAMS, "parameter packing");
 constexpr int kMaxMembers = 64;
 constexpr int kRows = 128;          // tile rows = TMEM lanes
 // 16 warps per tile: warp w reads TMEM lanes 32 (w % 4) .. + 31 (the lanes
-// its rank in a group of four may access) and the columns of quarter w / 4
+// its rank in a group of four may access) and 16 columns, from 16 (w / 4)
 constexpr int kThreads = 512;
-constexpr int kQuarter = 64;        // accumulator columns per warp
-constexpr int kKC = 128;            // K columns staged per round
-constexpr int kSmemA = kRows * kKC * 2;     // 32 KB
-constexpr int kSmemB = H * kKC * 2;         // 64 KB
+constexpr int kQuarter = 64;        // columns of D (N) per tile
+constexpr int kSplit = H / kQuarter;        // tiles side by side
+constexpr int kCols = kQuarter / 4;         // accumulator columns per warp
+constexpr int kKC = 256;            // K columns staged per round
+constexpr int kSmemA = kRows * kKC * 2;     // 64 KB
+constexpr int kSmemB = kQuarter * kKC * 2;  // 32 KB
 // Shared memory of a tile CTA: the operand buffers A and B from 0; after the
 // last product, the forward epilogue's H2 tile over them (rows padded to
-// 260 floats so that 8 rows' 16-byte accesses hit distinct banks); then the
-// small parameter vectors, the row partial sums, and the barrier.  Each tile
-// CTA takes the largest allocation, so one tile CTA runs per SM and its 256
-// tensor-memory columns never wait for another's.
-constexpr int kH2Stride = H + 4;
-constexpr int kSmemPrm = kRows * kH2Stride * 4;            // W1, b1, b2, W3, b3
-constexpr int kNPrm = H * NI + H + H + NO * H + NO;
+// 68 floats so that 8 rows' 16-byte accesses hit distinct banks); then the
+// small parameter vectors, the row partial sums, and the barrier.
+constexpr int kH2Stride = kQuarter + 4;
+constexpr int kSmemPrm = kSmemA + kSmemB;                  // W1, b1, b2, W3, b3 (own quarters)
+constexpr int kNPrm = kQuarter * (NI + 1 + 1 + NO) + NO;
 constexpr int kSmemPart = kSmemPrm + (kNPrm * 4 + 15) / 16 * 16;  // [4][kRows][2]
-constexpr int kSmemBar = kSmemPart + 4 * kRows * 2 * 4;
-constexpr int kSmemTile = 232448;
-static_assert(kSmemA + kSmemB <= kSmemPrm && kSmemBar + 16 <= kSmemTile, "tile shared memory");
-constexpr int kTmemCols = 256;      // FP32 accumulator columns (N)
+constexpr int kSmemBar = kSmemPart + kSplit * kRows * 2 * 4;
+constexpr int kSmemTile = kSmemBar + 16;
+static_assert(kRows * kH2Stride * 4 <= kSmemPrm && 2 * (kSmemTile + 1024) <= 228 * 1024,
+              "tile shared memory: two CTAs per SM");
 constexpr uint32_t kDrainLimit = 1u << 22;  // second wait, after a timeout
 
 // ---- tcgen05 / mbarrier wrappers -------------------------------------------
@@ -112,7 +121,6 @@ constexpr uint32_t idesc_bf16_f32(int M, int N)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
            ((uint32_t)(M >> 4) << 24);
 }
-constexpr uint32_t kIdesc = idesc_bf16_f32(kRows, H);
 
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t ncols)
 {
@@ -199,35 +207,34 @@ __device__ __forceinline__ uint32_t core_off(int R, int r, int c8)
     return (uint32_t)(c8 * R * 16 + (r >> 3) * 128 + (r & 7) * 16);
 }
 
-// Item i of a staging round: row r and 8-column group c8 of the kKC
-// columns; eight consecutive items fill one core matrix (128 contiguous
-// bytes of shared memory, 16 B from each of 8 rows).
-__device__ __forceinline__ void stage_item(int i, int &r, int &c8)
+// Item i of a staging round of `c8n` 8-column groups: row r and group c8;
+// eight consecutive items fill one core matrix (128 contiguous bytes of
+// shared memory, 16 B from each of 8 rows).
+__device__ __forceinline__ void stage_item(int i, int c8n, int &r, int &c8)
 {
-    constexpr int c8n = kKC / 8;
     c8 = (i >> 3) % c8n;
     r = (i >> 3) / c8n * 8 + (i & 7);
 }
 
-// Rows [r0, r0 + R) x columns [k0, k0 + kKC) of a row-major bf16 matrix
+// Rows [r0, r0 + R) x columns [k0, k0 + KC) of a row-major bf16 matrix
 // (leading dimension ld, a multiple of 8) into the canonical layout at s:
 // every thread issues all its loads before its first store.
-template <int R>
-__device__ __forceinline__ void stage_bf16(uint8_t *s, const __nv_bfloat16 *__restrict__ g,
-                                           long long ld, int r0, int k0)
+template <int R, int KC>
+__device__ __forceinline__ void stage_bf16(uint8_t *s, const __nv_bfloat16 *g, long long ld, int r0,
+                                           int k0)
 {
-    constexpr int per = R * (kKC / 8) / kThreads;
+    constexpr int per = R * (KC / 8) / kThreads;
     uint4 v[per];
 #pragma unroll
     for (int u = 0; u < per; ++u) {
         int r, c8;
-        stage_item(threadIdx.x + u * kThreads, r, c8);
+        stage_item(threadIdx.x + u * kThreads, KC / 8, r, c8);
         v[u] = *reinterpret_cast<const uint4 *>(g + (long long)(r0 + r) * ld + k0 + c8 * 8);
     }
 #pragma unroll
     for (int u = 0; u < per; ++u) {
         int r, c8;
-        stage_item(threadIdx.x + u * kThreads, r, c8);
+        stage_item(threadIdx.x + u * kThreads, KC / 8, r, c8);
         *reinterpret_cast<uint4 *>(s + core_off(R, r, c8)) = v[u];
     }
 }
@@ -249,7 +256,7 @@ struct NetView {
     float *Y, *dY;                         // Bmax x NO
     double *lrow;                          // per-row loss terms
     long long Bmax;
-    int *err;                              // set when a tensor-core wait ran out
+    int *err;                              // pinned host word, set when a tensor-core wait ran out
     uint32_t limit;                        // polls before that wait gives up
 };
 
@@ -258,17 +265,18 @@ struct Tile {
     uint32_t bar, tmem;
 };
 
-// Warp 0 allocates the accumulator's tensor-memory columns; thread 0
-// initialises the completion barrier.
-__device__ __forceinline__ Tile tile_setup(uint8_t *smem)
+// Warp 0 allocates the accumulator's N tensor-memory columns; thread 0
+// initialises the completion barrier (at `bar`, 16 bytes, in smem).
+template <int N>
+__device__ __forceinline__ Tile tile_setup(uint8_t *smem, int offB, int offBar)
 {
     Tile t;
     t.sA = smem;
-    t.sB = smem + kSmemA;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kSmemBar);
+    t.sB = smem + offB;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + offBar);
     uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 1);
     t.bar = smem_u32(bar);
-    if (threadIdx.x < 32) tmem_alloc(smem_u32(slot), kTmemCols);
+    if (threadIdx.x < 32) tmem_alloc(smem_u32(slot), N);
     if (threadIdx.x == 0) bar_init(t.bar, 1);
     tc_fence_before();
     __syncthreads();
@@ -277,52 +285,83 @@ __device__ __forceinline__ Tile tile_setup(uint8_t *smem)
     return t;
 }
 
-__device__ __forceinline__ void tile_teardown(const Tile &t)
+template <int N> __device__ __forceinline__ void tile_teardown(const Tile &t)
 {
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x < 32) tmem_dealloc(t.tmem, kTmemCols);
+    if (threadIdx.x < 32) tmem_dealloc(t.tmem, N);
 }
 
-// D (TMEM, 128 x 256 FP32) = A (128 x K) B (256 x K)^T, K a multiple of
-// kKC, in rounds of kKC columns: stage_a(k0) and stage_b(k0) fill the
-// operand buffers, thread 0 issues kKC / 16 products and commits them, and
-// all threads wait for them before the buffers are refilled.  Returns false,
-// in every thread alike, when a wait ran out: the error flag is set and the
-// products in flight are waited for (again with a limit) so that the tensor
-// memory can be released.
-template <class SA, class SB>
-__device__ __forceinline__ bool tile_product(const Tile &t, int K, uint32_t limit, int *err,
-                                             SA stage_a, SB stage_b)
+// The products of `kc` staged columns of K (a multiple of 16) into D, added to
+// it if `accumulate`, and their commit.  One thread.
+template <int N>
+__device__ __forceinline__ void issue_products(const Tile &t, int kc, bool accumulate)
 {
-    uint32_t phase = 0;
-    for (int k0 = 0; k0 < K; k0 += kKC) {
-        stage_a(k0);
-        stage_b(k0);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // stores -> tensor cores
+    constexpr uint32_t kIdesc = idesc_bf16_f32(kRows, N);
+    tc_fence_after();
+    const uint32_t a0 = smem_u32(t.sA), b0 = smem_u32(t.sB);
+    for (int kk = 0; kk < kc; kk += 16) {
+        const uint64_t da = smem_desc(a0 + (uint32_t)(kk >> 3) * kRows * 16, kRows * 16, 128);
+        const uint64_t db = smem_desc(b0 + (uint32_t)(kk >> 3) * N * 16, N * 16, 128);
+        mma_bf16(t.tmem, da, db, kIdesc, accumulate || kk > 0 ? 1u : 0u);
+    }
+    mma_commit(t.bar);
+}
+
+// Waits for the committed products.  Returns false, in every thread alike,
+// when the wait ran out: the error flag is set and the products in flight are
+// waited for (again with a limit) so that the tensor memory can be released.
+__device__ __forceinline__ bool wait_products(const Tile &t, uint32_t phase, uint32_t limit, int *err)
+{
+    const bool ok = __syncthreads_and(bar_wait(t.bar, phase, limit));
+    if (!ok) {
+        if (threadIdx.x == 0) *reinterpret_cast<volatile int *>(err) = 1;
+        bar_wait(t.bar, phase, kDrainLimit);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            tc_fence_after();
-            const uint32_t a0 = smem_u32(t.sA), b0 = smem_u32(t.sB);
-#pragma unroll
-            for (int kk = 0; kk < kKC; kk += 16) {
-                const uint64_t da = smem_desc(a0 + (uint32_t)(kk >> 3) * kRows * 16, kRows * 16, 128);
-                const uint64_t db = smem_desc(b0 + (uint32_t)(kk >> 3) * H * 16, H * 16, 128);
-                mma_bf16(t.tmem, da, db, kIdesc, (k0 + kk) > 0 ? 1u : 0u);
-            }
-            mma_commit(t.bar);
-        }
-        const bool ok = __syncthreads_and(bar_wait(t.bar, phase, limit));
-        if (!ok) {
-            if (threadIdx.x == 0) atomicExch(err, 1);
-            bar_wait(t.bar, phase, kDrainLimit);
-            __syncthreads();
-            return false;
-        }
-        phase ^= 1u;
+        return false;
     }
     tc_fence_after();
     return true;
+}
+
+// D (TMEM, 128 x 64 FP32) = A (128 x K) B (64 x K)^T, K a multiple of 128:
+// rows [ra, ra + 128) of a (leading dimension lda) and [rb, rb + 64) of b, in
+// rounds of kKC columns (the last may have half as many): stage, one thread
+// issues, all threads wait before the buffers are refilled.
+__device__ __forceinline__ bool tile_product(const Tile &t, int K, uint32_t limit, int *err,
+                                             const __nv_bfloat16 *a, long long lda, int ra,
+                                             const __nv_bfloat16 *b, long long ldb, int rb)
+{
+    uint32_t phase = 0;
+    for (int k0 = 0; k0 < K; k0 += kKC) {
+        const int kc = K - k0 < kKC ? K - k0 : kKC;
+        if (kc == kKC) {
+            stage_bf16<kRows, kKC>(t.sA, a, lda, ra, k0);
+            stage_bf16<kQuarter, kKC>(t.sB, b, ldb, rb, k0);
+        } else {
+            stage_bf16<kRows, kKC / 2>(t.sA, a, lda, ra, k0);
+            stage_bf16<kQuarter, kKC / 2>(t.sB, b, ldb, rb, k0);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // stores -> tensor cores
+        __syncthreads();
+        if (threadIdx.x == 0) issue_products<kQuarter>(t, kc, k0 > 0);
+        if (!wait_products(t, phase, limit, err)) return false;
+        phase ^= 1u;
+    }
+    return true;
+}
+
+// The four CTAs of a cluster meet; what each wrote before, the others see.
+__device__ __forceinline__ void cluster_meet()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address of shared-memory address `a` in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t peer(uint32_t a, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
 }
 
 __device__ __forceinline__ void store16(float *p, const float (&v)[16])
@@ -333,122 +372,151 @@ __device__ __forceinline__ void store16(float *p, const float (&v)[16])
 }
 
 // This thread's place in the epilogue: tile row r (TMEM lane 32 (w % 4) +
-// lane of warp w) and the first of its 64 columns, j0 = 64 (w / 4).
+// lane of warp w) and the first of its 16 columns, c = 16 (w / 4).
 struct Seat {
-    int r, q, j0;
-    uint32_t ta;  // tensor-memory address of (row r, column j0)
+    int r, c;
+    uint32_t ta;  // tensor-memory address of (row r, column c)
 };
 __device__ __forceinline__ Seat seat(const Tile &t)
 {
     Seat s;
     const int w = threadIdx.x >> 5, g = w & 3;
-    s.q = w >> 2;
+    s.c = (w >> 2) * kCols;
     s.r = 32 * g + (threadIdx.x & 31);
-    s.j0 = s.q * kQuarter;
-    s.ta = t.tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)s.j0;
+    s.ta = t.tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)s.c;
     return s;
 }
 
 // Forward pass of batch rows [m0, m0 + 128) of member blockIdx.y (rows past
-// nb are padding: H1 = 0, no loss, dY = 0).  BACK: also the quantities the
-// backward pass reads (H1 in FP32 and as bf16 H1^T, H2, dY, the row loss,
-// dZ2 in FP32, bf16 and bf16 transposed).  X and T: row-major inputs and
-// targets, member e's at X + e xs and T + e ts.  Each row's two outputs are
-// summed over its four column quarters, then added to b3 in quarter order.
+// nb are padding: H1 = 0, no loss, dY = 0) by a cluster of four CTAs: CTA q
+// computes columns 64 q .. 64 q + 63 of H1, for all four, and of H2.  BACK:
+// also the quantities the backward pass reads (H1 in FP32 and as bf16 H1^T,
+// H2, dY, the row loss, dZ2 in FP32, bf16 and bf16 transposed).  X and T:
+// row-major inputs and targets, member e's at X + e xs and T + e ts.  Each
+// row's two outputs are summed over a quarter's 64 columns in order, then the
+// four quarters are added to b3 in order.
 template <bool BACK>
-__global__ void __launch_bounds__(kThreads, 1)
-    forward_kernel(NetView v, const float *__restrict__ X, long long xs,
-                   const float *__restrict__ T, long long ts, int nb, int Bp)
+__global__ void __launch_bounds__(kThreads, 2) __cluster_dims__(kSplit, 1, 1)
+    forward_kernel(NetView v, const float *X, long long xs, const float *T, long long ts, int nb,
+                   int Bp)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int e = blockIdx.y, m0 = blockIdx.x * kRows;
-    const float *__restrict__ P = v.P + (long long)e * NPARAM;
+    const int e = blockIdx.y, q = blockIdx.x % kSplit, m0 = blockIdx.x / kSplit * kRows;
+    const int j0 = q * kQuarter;  // first column of this CTA's quarter
+    const float *P = v.P + (long long)e * NPARAM;
     X += (long long)e * xs;
     const long long act = (long long)e * v.Bmax * H;
     const __nv_bfloat16 *W2b = v.W2b + (long long)e * H * H;
-    // W1, b1 (contiguous in P), then b2, W3, b3 (contiguous in P)
-    float *prm = reinterpret_cast<float *>(smem + kSmemPrm);
-    const float *sW1 = prm, *sB1 = prm + H * NI, *sB2 = sB1 + H, *sW3 = sB2 + H, *sB3 = sW3 + NO * H;
-    for (int i = threadIdx.x; i < H * NI + H; i += kThreads) prm[i] = P[OFF_W1 + i];
-    for (int i = threadIdx.x; i < H + NO * H + NO; i += kThreads) prm[H * NI + H + i] = P[OFF_B2 + i];
-    const Tile t = tile_setup(smem);  // (its barrier also publishes prm)
+    float *sW1 = reinterpret_cast<float *>(smem + kSmemPrm), *sB1 = sW1 + kQuarter * NI,
+          *sB2 = sB1 + kQuarter, *sW3 = sB2 + kQuarter, *sB3 = sW3 + NO * kQuarter;
+    const Tile t = tile_setup<kQuarter>(smem, kSmemA, kSmemBar);
+    cx::pass_wait();
+    for (int i = threadIdx.x; i < kQuarter * NI; i += kThreads) sW1[i] = P[OFF_W1 + j0 * NI + i];
+    for (int i = threadIdx.x; i < kQuarter; i += kThreads) {
+        sB1[i] = P[OFF_B1 + j0 + i];
+        sB2[i] = P[OFF_B2 + j0 + i];
+        sW3[i] = P[OFF_W3 + j0 + i];
+        sW3[kQuarter + i] = P[OFF_W3 + H + j0 + i];
+        if (i < NO) sB3[i] = P[OFF_B3 + i];
+    }
+    stage_bf16<kQuarter, H>(t.sB, W2b, H, j0, 0);
+    __syncthreads();
+    cluster_meet();  // every CTA of the cluster runs: its shared memory may be written
 
-    // A = bf(H1) for the tile's rows, computed while it is staged
-    auto stage_a = [&](int k0) {
-        constexpr int per = kRows * (kKC / 8) / kThreads;
+    // A = bf(H1) for the tile's rows: this quarter's columns into all four CTAs
+    constexpr int per = kRows * (kQuarter / 8) / kThreads;
 #pragma unroll 1
-        for (int u = 0; u < per; ++u) {
-            int r, c8;
-            stage_item(threadIdx.x + u * kThreads, r, c8);
-            const int b = m0 + r, j0 = k0 + c8 * 8;
-            float h[8];
-            if (b < nb) {
-                const float4 x = *reinterpret_cast<const float4 *>(X + (long long)b * NI);
+    for (int u = 0; u < per; ++u) {
+        int r, c8;
+        stage_item(threadIdx.x + u * kThreads, kQuarter / 8, r, c8);
+        const int b = m0 + r, jq = c8 * 8, j = j0 + jq;
+        float h[8];
+        if (b < nb) {
+            const float4 x = *reinterpret_cast<const float4 *>(X + (long long)b * NI);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 w = *reinterpret_cast<const float4 *>(sW1 + (j0 + q) * NI);
-                    float z = sB1[j0 + q];
-                    z += w.x * x.x;
-                    z += w.y * x.y;
-                    z += w.z * x.z;
-                    z += w.w * x.w;
-                    h[q] = tanhf(z);
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) h[q] = 0.f;
+            for (int i = 0; i < 8; ++i) {
+                const float4 w = *reinterpret_cast<const float4 *>(sW1 + (jq + i) * NI);
+                float z = sB1[jq + i];
+                z += w.x * x.x;
+                z += w.y * x.y;
+                z += w.z * x.z;
+                z += w.w * x.w;
+                h[i] = tanhf(z);
             }
-            *reinterpret_cast<uint4 *>(t.sA + core_off(kRows, r, c8)) =
-                make_uint4(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]), pack_bf16(h[4], h[5]),
-                           pack_bf16(h[6], h[7]));
-            if (BACK) {
-                float *hf = v.H1f + act + (long long)b * H + j0;
-                *reinterpret_cast<float4 *>(hf) = make_float4(h[0], h[1], h[2], h[3]);
-                *reinterpret_cast<float4 *>(hf + 4) = make_float4(h[4], h[5], h[6], h[7]);
+        } else {
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    v.H1T[act + (long long)(j0 + q) * Bp + b] = __float2bfloat16_rn(h[q]);
-            }
+            for (int i = 0; i < 8; ++i) h[i] = 0.f;
         }
-    };
-    auto stage_b = [&](int k0) { stage_bf16<H>(t.sB, W2b, H, 0, k0); };
-    const bool ok = tile_product(t, H, v.limit, v.err, stage_a, stage_b);
+        const uint4 p = make_uint4(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]), pack_bf16(h[4], h[5]),
+                                   pack_bf16(h[6], h[7]));
+        const uint32_t at = smem_u32(t.sA) + core_off(kRows, r, j / 8);
+#pragma unroll
+        for (uint32_t c = 0; c < kSplit; ++c)
+            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(peer(at, c)), "r"(p.x),
+                         "r"(p.y), "r"(p.z), "r"(p.w)
+                         : "memory");
+        if (BACK) {
+            float *hf = v.H1f + act + (long long)b * H + j;
+            *reinterpret_cast<float4 *>(hf) = make_float4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<float4 *>(hf + 4) = make_float4(h[4], h[5], h[6], h[7]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                v.H1T[act + (long long)(j + i) * Bp + b] = __float2bfloat16_rn(h[i]);
+        }
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");  // stores -> the four CTAs' tensor cores
+    cluster_meet();
+    asm volatile("fence.proxy.async;" ::: "memory");
+    if (threadIdx.x == 0) issue_products<kQuarter>(t, H, false);
+    // (a CTA whose wait ran out still meets the others)
+    const bool ok = wait_products(t, 0, v.limit, v.err);
 
+    const Seat st = seat(t);
+    const int b = m0 + st.r;
+    float *h2s = reinterpret_cast<float *>(smem);  // over the operands: the products are complete
+    float *part = reinterpret_cast<float *>(smem + kSmemPart);  // [quarter][row][2]
+    float a[kCols];
+    const long long o = act + (long long)b * H + j0 + st.c;
     if (ok) {
-        const Seat st = seat(t);
-        const int b = m0 + st.r;
-        // the products are complete: H2 may overwrite the operand buffers
-        float *h2s = reinterpret_cast<float *>(smem) + st.r * kH2Stride + st.j0;
-        float *part = reinterpret_cast<float *>(smem + kSmemPart);  // [4][kRows][2]
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll 1
-        for (int c = 0; c < kQuarter / 16; ++c) {
-            float a[16];
-            tmem_ld16(st.ta + 16 * c, a);
+        tmem_ld16(st.ta, a);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int j = st.j0 + 16 * c + q;
-                const float h = tanhf(a[q] + sB2[j]);
-                s0 += sW3[j] * h;
-                s1 += sW3[H + j] * h;
-                a[q] = h;
-            }
-            if (BACK) {
-                store16(v.H2 + act + (long long)b * H + st.j0 + 16 * c, a);
-                store16(h2s + 16 * c, a);
-            }
+        for (int i = 0; i < kCols; ++i) a[i] = tanhf(a[i] + sB2[st.c + i]);
+        store16(h2s + st.r * kH2Stride + st.c, a);
+        if (BACK) store16(v.H2 + o, a);
+    }
+    __syncthreads();
+    if (threadIdx.x < kRows) {
+        const int r = threadIdx.x;
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll 4
+        for (int j = 0; j < kQuarter; j += 4) {
+            const float4 h = *reinterpret_cast<const float4 *>(h2s + r * kH2Stride + j);
+            s0 += sW3[j] * h.x;
+            s1 += sW3[kQuarter + j] * h.x;
+            s0 += sW3[j + 1] * h.y;
+            s1 += sW3[kQuarter + j + 1] * h.y;
+            s0 += sW3[j + 2] * h.z;
+            s1 += sW3[kQuarter + j + 2] * h.z;
+            s0 += sW3[j + 3] * h.w;
+            s1 += sW3[kQuarter + j + 3] * h.w;
         }
-        part[(st.q * kRows + st.r) * 2] = s0;
-        part[(st.q * kRows + st.r) * 2 + 1] = s1;
-        __syncthreads();
+        const uint32_t at = smem_u32(part + (q * kRows + r) * 2);
+#pragma unroll
+        for (uint32_t c = 0; c < kSplit; ++c)
+            asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(peer(at, c)), "f"(s0), "f"(s1)
+                         : "memory");
+    }
+    cluster_meet();  // the last access to another CTA's shared memory
+    if (ok) {
         float y0 = sB3[0], y1 = sB3[1];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < kSplit; ++k) {
             y0 += part[(k * kRows + st.r) * 2];
             y1 += part[(k * kRows + st.r) * 2 + 1];
         }
         const long long yo = (long long)e * v.Bmax * NO + (long long)b * NO;
-        if (st.q == 0) {
+        const bool first = q == 0 && st.c == 0;
+        if (first) {
             v.Y[yo] = y0;
             v.Y[yo + 1] = y1;
         }
@@ -460,105 +528,180 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float r0 = y0 - T[(long long)b * NO], r1 = y1 - T[(long long)b * NO + 1];
                 d0 = r0 / (float)nb;
                 d1 = r1 / (float)nb;
-                l += 0.5 * (double)r0 * (double)r0;
-                l += 0.5 * (double)r1 * (double)r1;
+                if (first) {
+                    l += 0.5 * (double)r0 * (double)r0;
+                    l += 0.5 * (double)r1 * (double)r1;
+                }
             }
-            if (st.q == 0) {
+            if (first) {
                 v.dY[yo] = d0;
                 v.dY[yo + 1] = d1;
                 v.lrow[(long long)e * v.Bmax + b] = l;
             }
-#pragma unroll 1
-            for (int c = 0; c < kQuarter / 16; ++c) {
-                float a[16];
 #pragma unroll
-                for (int q = 0; q < 16; q += 4) {
-                    const float4 h4 = *reinterpret_cast<const float4 *>(h2s + 16 * c + q);
-                    a[q] = h4.x;
-                    a[q + 1] = h4.y;
-                    a[q + 2] = h4.z;
-                    a[q + 3] = h4.w;
-                }
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int j = st.j0 + 16 * c + q;
-                    const float h = a[q];
-                    float s = 0.f;
-                    s += d0 * sW3[j];
-                    s += d1 * sW3[H + j];
-                    a[q] = s * (1.f - h * h);
-                    v.dZ2T[act + (long long)j * Bp + b] = __float2bfloat16_rn(a[q]);
-                }
-                const long long o = act + (long long)b * H + st.j0 + 16 * c;
-                store16(v.dZ2 + o, a);
-                uint4 *pb = reinterpret_cast<uint4 *>(v.dZ2b + o);
-                pb[0] = make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]),
-                                   pack_bf16(a[6], a[7]));
-                pb[1] = make_uint4(pack_bf16(a[8], a[9]), pack_bf16(a[10], a[11]),
-                                   pack_bf16(a[12], a[13]), pack_bf16(a[14], a[15]));
+            for (int i = 0; i < kCols; ++i) {
+                const int j = st.c + i;
+                const float h = a[i];
+                float s = 0.f;
+                s += d0 * sW3[j];
+                s += d1 * sW3[kQuarter + j];
+                a[i] = s * (1.f - h * h);
+                v.dZ2T[act + (long long)(j0 + j) * Bp + b] = __float2bfloat16_rn(a[i]);
             }
+            store16(v.dZ2 + o, a);
+            uint4 *pb = reinterpret_cast<uint4 *>(v.dZ2b + o);
+            pb[0] = make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]),
+                               pack_bf16(a[6], a[7]));
+            pb[1] = make_uint4(pack_bf16(a[8], a[9]), pack_bf16(a[10], a[11]),
+                               pack_bf16(a[12], a[13]), pack_bf16(a[14], a[15]));
         }
     }
-    tile_teardown(t);
+    tile_teardown<kQuarter>(t);
 }
 
-// Backward products of member blockIdx.y.  Tiles 0 .. Bp/128 - 1: dH1 for
-// batch rows [128 t, 128 t + 128) = bf(dZ2) rows times bf(W2) (B operand:
-// the rows of W2^T), epilogue dZ1 = dH1 (1 - H1^2).  The last two tiles:
-// dW2 rows [128 u, 128 u + 128) = bf(dZ2)^T rows times bf(H1) (B operand:
-// the rows of H1^T), over K = Bp.
-__global__ void __launch_bounds__(kThreads, 1) backward_kernel(NetView v, int Bp)
+// Forward pass alone on many rows: batch rows [128 i, 128 i + 128) of member
+// blockIdx.y, i = blockIdx.x, all 256 columns in one CTA, whose H1 needs no
+// other CTA.  With more tiles than the GPU holds at a time throughput counts,
+// not a tile's latency: a call of 8 members x 8192 rows takes 99 us (clusters
+// 125; with the whole shared memory per CTA, one per SM, 104), while at 8 x 1024
+// rows the clusters take 41 (51).  Same sums in the same order as the clusters
+// (a thread sums one quarter of a row).
+constexpr int kWideKC = 128;
+constexpr int kWideA = kRows * kWideKC * 2, kWideB = H * kWideKC * 2;
+constexpr int kWidePrm = kWideA + kWideB;  // W1, b1, b2, W3, b3
+constexpr int kWidePart = kWidePrm + ((H * NI + H + H + NO * H + NO) * 4 + 15) / 16 * 16;
+constexpr int kWideBar = kWidePart + 4 * kRows * 2 * 4;
+constexpr int kWideSmem = kWideBar + 16;
+static_assert(2 * (kWideSmem + 1024) <= 228 * 1024, "two CTAs per SM (and 2 x 256 columns of TMEM)");
+__global__ void __launch_bounds__(kThreads, 2)
+    forward_wide_kernel(NetView v, const float *X, int nb)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int e = blockIdx.y, nt = Bp / kRows;
-    const long long act = (long long)e * v.Bmax * H;
-    const Tile t = tile_setup(smem);
-    if ((int)blockIdx.x < nt) {
-        const int m0 = blockIdx.x * kRows;
-        const __nv_bfloat16 *A = v.dZ2b + act, *B = v.W2T + (long long)e * H * H;
-        const bool ok = tile_product(
-            t, H, v.limit, v.err, [&](int k0) { stage_bf16<kRows>(t.sA, A, H, m0, k0); },
-            [&](int k0) { stage_bf16<H>(t.sB, B, H, 0, k0); });
-        if (ok) {
-            const Seat st = seat(t);
-            const long long row = act + (long long)(m0 + st.r) * H + st.j0;
+    const int e = blockIdx.y, m0 = blockIdx.x * kRows;
+    const float *P = v.P + (long long)e * NPARAM;
+    const __nv_bfloat16 *W2b = v.W2b + (long long)e * H * H;
+    // W1, b1 (contiguous in P), then b2, W3, b3 (contiguous in P)
+    float *prm = reinterpret_cast<float *>(smem + kWidePrm);
+    const float *sW1 = prm, *sB1 = prm + H * NI, *sB2 = sB1 + H, *sW3 = sB2 + H, *sB3 = sW3 + NO * H;
+    const Tile t = tile_setup<H>(smem, kWideA, kWideBar);
+    cx::pass_wait();
+    for (int i = threadIdx.x; i < H * NI + H; i += kThreads) prm[i] = P[OFF_W1 + i];
+    for (int i = threadIdx.x; i < H + NO * H + NO; i += kThreads) prm[H * NI + H + i] = P[OFF_B2 + i];
+    __syncthreads();
+    bool ok = true;
+    for (int k0 = 0; k0 < H && ok; k0 += kWideKC) {
+        constexpr int per = kRows * (kWideKC / 8) / kThreads;
+        stage_bf16<H, kWideKC>(t.sB, W2b, H, 0, k0);
 #pragma unroll 1
-            for (int c = 0; c < kQuarter / 16; ++c) {
-                float a[16];
-                tmem_ld16(st.ta + 16 * c, a);
+        for (int u = 0; u < per; ++u) {
+            int r, c8;
+            stage_item(threadIdx.x + u * kThreads, kWideKC / 8, r, c8);
+            const int b = m0 + r, j = k0 + c8 * 8;
+            float h[8];
+            if (b < nb) {
+                const float4 x = *reinterpret_cast<const float4 *>(X + (long long)b * NI);
 #pragma unroll
-                for (int q = 0; q < 16; q += 4) {
-                    const float4 h1 = *reinterpret_cast<const float4 *>(v.H1f + row + 16 * c + q);
-                    a[q] = a[q] * (1.f - h1.x * h1.x);
-                    a[q + 1] = a[q + 1] * (1.f - h1.y * h1.y);
-                    a[q + 2] = a[q + 2] * (1.f - h1.z * h1.z);
-                    a[q + 3] = a[q + 3] * (1.f - h1.w * h1.w);
+                for (int i = 0; i < 8; ++i) {
+                    const float4 w = *reinterpret_cast<const float4 *>(sW1 + (j + i) * NI);
+                    float z = sB1[j + i];
+                    z += w.x * x.x;
+                    z += w.y * x.y;
+                    z += w.z * x.z;
+                    z += w.w * x.w;
+                    h[i] = tanhf(z);
                 }
-                store16(v.dZ1 + row + 16 * c, a);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) h[i] = 0.f;
+            }
+            *reinterpret_cast<uint4 *>(t.sA + core_off(kRows, r, c8)) =
+                make_uint4(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]), pack_bf16(h[4], h[5]),
+                           pack_bf16(h[6], h[7]));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // stores -> tensor cores
+        __syncthreads();
+        if (threadIdx.x == 0) issue_products<H>(t, kWideKC, k0 > 0);
+        ok = wait_products(t, (k0 / kWideKC) & 1, v.limit, v.err);
+    }
+    if (ok) {
+        // warp w: rows 32 (w % 4) .. + 31, columns of quarter w / 4
+        const int w = threadIdx.x >> 5, q = w >> 2, r = 32 * (w & 3) + (threadIdx.x & 31);
+        const uint32_t ta = t.tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(q * kQuarter);
+        float *part = reinterpret_cast<float *>(smem + kWidePart);  // [quarter][row][2]
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll 1
+        for (int c = 0; c < kQuarter; c += 16) {
+            float a[16];
+            tmem_ld16(ta + c, a);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int j = q * kQuarter + c + i;
+                const float h = tanhf(a[i] + sB2[j]);
+                s0 += sW3[j] * h;
+                s1 += sW3[H + j] * h;
             }
         }
-    } else {
-        const int i0 = (blockIdx.x - nt) * kRows;
-        const __nv_bfloat16 *A = v.dZ2T + act, *B = v.H1T + act;
-        const bool ok = tile_product(
-            t, Bp, v.limit, v.err, [&](int k0) { stage_bf16<kRows>(t.sA, A, Bp, i0, k0); },
-            [&](int k0) { stage_bf16<H>(t.sB, B, Bp, 0, k0); });
-        if (ok) {
-            // a member's block starts at e * NPARAM floats, a multiple of 8
-            // bytes only: pairs, not quads
-            const Seat st = seat(t);
-            float *g = v.G + (long long)e * NPARAM + OFF_W2 + (long long)(i0 + st.r) * H + st.j0;
-#pragma unroll 1
-            for (int c = 0; c < kQuarter / 16; ++c) {
-                float a[16];
-                tmem_ld16(st.ta + 16 * c, a);
+        part[(q * kRows + r) * 2] = s0;
+        part[(q * kRows + r) * 2 + 1] = s1;
+        __syncthreads();
+        if (q == 0) {
+            float y0 = sB3[0], y1 = sB3[1];
 #pragma unroll
-                for (int q = 0; q < 16; q += 2)
-                    *reinterpret_cast<float2 *>(g + 16 * c + q) = make_float2(a[q], a[q + 1]);
+            for (int k = 0; k < 4; ++k) {
+                y0 += part[(k * kRows + r) * 2];
+                y1 += part[(k * kRows + r) * 2 + 1];
             }
+            const long long yo = (long long)e * v.Bmax * NO + (long long)(m0 + r) * NO;
+            v.Y[yo] = y0;
+            v.Y[yo + 1] = y1;
         }
     }
-    tile_teardown(t);
+    tile_teardown<H>(t);
+}
+
+// Backward products of member blockIdx.y, columns 64 q .. 64 q + 63 of each.
+// Tiles 0 .. Bp/128 - 1: dH1 for batch rows [128 t, 128 t + 128) = bf(dZ2) rows
+// times bf(W2) (B operand: the rows of W2^T), epilogue dZ1 = dH1 (1 - H1^2).
+// The last two tiles: dW2 rows [128 u, 128 u + 128) = bf(dZ2)^T rows times
+// bf(H1) (B operand: the rows of H1^T), over K = Bp.
+__global__ void __launch_bounds__(kThreads, 2) backward_kernel(NetView v, int Bp)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int e = blockIdx.y, nt = Bp / kRows, tile = blockIdx.x / kSplit;
+    const int j0 = blockIdx.x % kSplit * kQuarter;
+    const long long act = (long long)e * v.Bmax * H;
+    const Tile t = tile_setup<kQuarter>(smem, kSmemA, kSmemBar);
+    cx::pass_wait();
+    const Seat st = seat(t);
+    float a[kCols];
+    if (tile < nt) {
+        const int m0 = tile * kRows;
+        if (tile_product(t, H, v.limit, v.err, v.dZ2b + act, H, m0, v.W2T + (long long)e * H * H, H, j0)) {
+            const long long o = act + (long long)(m0 + st.r) * H + j0 + st.c;
+            tmem_ld16(st.ta, a);
+#pragma unroll
+            for (int i = 0; i < kCols; i += 4) {
+                const float4 h1 = *reinterpret_cast<const float4 *>(v.H1f + o + i);
+                a[i] = a[i] * (1.f - h1.x * h1.x);
+                a[i + 1] = a[i + 1] * (1.f - h1.y * h1.y);
+                a[i + 2] = a[i + 2] * (1.f - h1.z * h1.z);
+                a[i + 3] = a[i + 3] * (1.f - h1.w * h1.w);
+            }
+            store16(v.dZ1 + o, a);
+        }
+    } else {
+        const int i0 = (tile - nt) * kRows;
+        if (tile_product(t, Bp, v.limit, v.err, v.dZ2T + act, Bp, i0, v.H1T + act, Bp, j0)) {
+            // a member's block starts at e * NPARAM floats, a multiple of 8
+            // bytes only: pairs, not quads
+            float *g = v.G + (long long)e * NPARAM + OFF_W2 + (long long)(i0 + st.r) * H + j0 + st.c;
+            tmem_ld16(st.ta, a);
+#pragma unroll
+            for (int i = 0; i < kCols; i += 2)
+                *reinterpret_cast<float2 *>(g + i) = make_float2(a[i], a[i + 1]);
+        }
+    }
+    tile_teardown<kQuarter>(t);
 }
 
 // Column sums over the nb valid rows of member blockIdx.y (padding rows
@@ -568,20 +711,19 @@ __global__ void __launch_bounds__(kThreads, 1) backward_kernel(NetView v, int Bp
 // 0 also sums db3 and the loss into loss_dst[e * loss_stride] (if given).
 constexpr int kSumCols = 16, kSumRows = 32;
 __global__ void __launch_bounds__(kSumCols *kSumRows)
-    column_sums(NetView v, const float *__restrict__ X, long long xs, int nb, double *loss_dst,
+    column_sums(NetView v, const float *X, long long xs, int nb, double *loss_dst,
                 long long loss_stride)
 {
     __shared__ float part[kSumRows][8][kSumCols];
     __shared__ float dpart[kSumRows * kSumCols][NO];
     __shared__ double lpart[kSumRows * kSumCols];
-    const int e = blockIdx.y, tx = threadIdx.x, ty = threadIdx.y;
+    const int e = blockIdx.y, tx = threadIdx.x % kSumCols, ty = threadIdx.x / kSumCols;
     const int j = blockIdx.x * kSumCols + tx;
     X += (long long)e * xs;
     const long long act = (long long)e * v.Bmax * H;
-    const float *__restrict__ H2 = v.H2 + act;
-    const float *__restrict__ dZ2 = v.dZ2 + act;
-    const float *__restrict__ dZ1 = v.dZ1 + act;
-    const float *__restrict__ dY = v.dY + (long long)e * v.Bmax * NO;
+    const float *H2 = v.H2 + act, *dZ2 = v.dZ2 + act, *dZ1 = v.dZ1 + act;
+    const float *dY = v.dY + (long long)e * v.Bmax * NO;
+    cx::pass_wait();
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // dW3 (2), db2, dW1 (4), db1
 #pragma unroll 4
     for (int b = ty; b < nb; b += kSumRows) {
@@ -647,11 +789,11 @@ __global__ void __launch_bounds__(kSumCols *kSumRows)
 
 // Adam (Kingma & Ba, 2015) on the FP32 master parameters of every member;
 // the threads of W2 entries also write the bf16 copies of W2 and W2^T.
-__global__ void adam_kernel(float *__restrict__ P, const float *__restrict__ G, float *__restrict__ M,
-                            float *__restrict__ V, __nv_bfloat16 *__restrict__ W2b,
-                            __nv_bfloat16 *__restrict__ W2T, long long n, float lr, float b1, float b2,
-                            float eps, float c1, float c2)
+__global__ void adam_kernel(float *P, const float *G, float *M, float *V, __nv_bfloat16 *W2b,
+                            __nv_bfloat16 *W2T, long long n, float lr, float b1, float b2, float eps,
+                            float c1, float c2)
 {
+    cx::pass_wait();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float g = G[i];
@@ -716,6 +858,7 @@ struct cx_mlp {
     int *err = nullptr;
     uint32_t limit = 1u << 22;  // polls before a tensor-core wait gives up
     long long adam_t = 0;
+    int num_sms = 1;
     cudaStream_t st = nullptr;
 };
 
@@ -726,9 +869,10 @@ void free_mlp(cx_mlp *m)
     if (!m) return;
     void *ptrs[] = {m->P, m->G, m->M, m->V, m->W2b, m->W2T, m->X, m->T, m->H1f, m->H2, m->dZ2,
                     m->dZ1, m->Y, m->dY, m->H1T, m->dZ2b, m->dZ2T, m->lrow, m->loss, m->dataX,
-                    m->dataT, m->losses, m->err};
+                    m->dataT, m->losses};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    if (m->err) cudaFreeHost(m->err);
     if (m->st) cudaStreamDestroy(m->st);
     delete m;
 }
@@ -766,28 +910,33 @@ cudaError_t run_pass(cx_mlp *m, const float *X, long long xs, const float *T, lo
 {
     const int Bp = (int)pad128(nb);
     const NetView v = view(m);
-    const dim3 grid(Bp / kRows, m->E);
-    if (!T) {
-        forward_kernel<false><<<grid, kThreads, kSmemTile, m->st>>>(v, X, xs, nullptr, 0, nb, Bp);
-        return cudaGetLastError();
-    }
-    forward_kernel<true><<<grid, kThreads, kSmemTile, m->st>>>(v, X, xs, T, ts, nb, Bp);
-    backward_kernel<<<dim3(Bp / kRows + H / kRows, m->E), kThreads, kSmemTile, m->st>>>(v, Bp);
-    column_sums<<<dim3(H / kSumCols, m->E), dim3(kSumCols, kSumRows), 0, m->st>>>(v, X, xs, nb, loss_dst,
-                                                                                   loss_stride);
-    return cudaGetLastError();
+    const dim3 grid(Bp / kRows * kSplit, m->E);
+    // clusters of four while the GPU holds all of them (two CTAs per SM), whole
+    // tiles beyond
+    if (!T && (long long)grid.x * m->E > 2LL * m->num_sms)
+        return cx::launch_pass(forward_wide_kernel, dim3(Bp / kRows, m->E), kThreads, kWideSmem, m->st, v,
+                               X, nb);
+    if (!T)
+        return cx::launch_pass(forward_kernel<false>, grid, kThreads, kSmemTile, m->st, v, X, xs, nullptr,
+                               0, nb, Bp);
+    cudaError_t e = cx::launch_pass(forward_kernel<true>, grid, kThreads, kSmemTile, m->st, v, X, xs, T,
+                                    ts, nb, Bp);
+    if (e == cudaSuccess)
+        e = cx::launch_pass(backward_kernel, dim3((Bp / kRows + H / kRows) * kSplit, m->E), kThreads,
+                            kSmemTile, m->st, v, Bp);
+    if (e == cudaSuccess)
+        e = cx::launch_pass(column_sums, dim3(H / kSumCols, m->E), kSumCols * kSumRows, 0, m->st, v, X,
+                            xs, nb, loss_dst, loss_stride);
+    return e;
 }
 
 // After the stream has drained: CX_ERR_TIMEOUT if a tile's wait ran out
 // (the flag is cleared for the next call).
 int check_waits(cx_mlp *m)
 {
-    int h = 0;
-    MX_CUDA(cudaMemcpyAsync(&h, m->err, sizeof h, cudaMemcpyDeviceToHost, m->st), "status download");
     MX_CUDA(cudaStreamSynchronize(m->st), "network synchronize");
-    if (h) {
-        MX_CUDA(cudaMemsetAsync(m->err, 0, sizeof(int), m->st), "status reset");
-        MX_CUDA(cudaStreamSynchronize(m->st), "network synchronize");
+    if (*m->err) {
+        *m->err = 0;
         return mfail(CX_ERR_TIMEOUT, "a tensor-core completion wait ran out");
     }
     return CX_OK;
@@ -831,12 +980,19 @@ int cx_mlp_create_members(int32_t max_batch, int32_t members, cx_mlp **out)
     A((void **)&m->dZ2T, E * Bp * H * 2);
     A((void **)&m->Y, E * Bp * NO * 4); A((void **)&m->dY, E * Bp * NO * 4);
     A((void **)&m->lrow, E * Bp * 8); A((void **)&m->loss, E * 8);
-    A((void **)&m->err, sizeof(int));
+    if (e == cudaSuccess) e = cudaMallocHost((void **)&m->err, sizeof(int));
+    if (e == cudaSuccess) *m->err = 0;
     const void *tiles[] = {(const void *)forward_kernel<false>, (const void *)forward_kernel<true>,
                            (const void *)backward_kernel};
     for (const void *f : tiles)
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTile);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void *)forward_wide_kernel,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmem);
+    int dev = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) {
         cudaGetLastError();
         free_mlp(m);
@@ -958,9 +1114,9 @@ int cx_mlp_train(cx_mlp *m, const float *x, const float *t, int32_t n, int32_t b
                 "training pass");
         m->adam_t += 1;
         const float c1 = 1.f - powf(b1, (float)m->adam_t), c2 = 1.f - powf(b2, (float)m->adam_t);
-        adam_kernel<<<(unsigned)((np + 255) / 256), 256, 0, m->st>>>(m->P, m->G, m->M, m->V, m->W2b,
-                                                                    m->W2T, np, lr, b1, b2, eps, c1, c2);
-        MX_CUDA(cudaGetLastError(), "optimiser launch");
+        MX_CUDA(cx::launch_pass(adam_kernel, (unsigned)((np + 255) / 256), 256, 0, m->st, m->P, m->G, m->M,
+                                m->V, m->W2b, m->W2T, np, lr, b1, b2, eps, c1, c2),
+                "optimiser launch");
     }
     if (loss_out && steps > 0)
         MX_CUDA(cudaMemcpyAsync(loss_out, m->losses, (size_t)(E * steps * 8), cudaMemcpyDeviceToHost, m->st),
