@@ -347,7 +347,11 @@ int cx_dt_limit(const cx_grid *g, const cx_params *p, double *limit)
 // FP64, one stage per pass: one-warp blocks of 128 columns, bound by the FP64
 // units, one per scheduler (four per SM).  A block of r rows costs about
 // r + 1/2 rows (it evaluates the y-faces behind its first row again), so the
-// height taken is the one with the least ceil(blocks / units) (r + 1/2).
+// height taken is the one with the least ceil(blocks / units) (r + 1/2); a
+// lone warp leaves its unit idle between dependent instructions and takes 1.4
+// times as long per row as two warps that share one (1024^2: 14 rows, one warp
+// per unit, 93.0 us per step; 7 rows, two, 90.6; 512^2: 4 rows 30.2, 2 rows
+// 27.4; 300^2: 16.3 and 14.9).
 static int auto_tile_rows_f64(const cx_ctx *c)
 {
     const long long tiles_x = ((long long)c->g.nx + 127) / 128, units = 4LL * c->num_sms;
@@ -356,7 +360,7 @@ static int auto_tile_rows_f64(const cx_ctx *c)
     for (long long r = 1; r <= 32; ++r) {
         const long long tiles_y = ((long long)c->g.ny + r - 1) / r;
         if (tiles_y > 65535) continue;
-        const double now = (double)((tiles_x * tiles_y + units - 1) / units) * ((double)r + 0.5);
+        const double now = cx::f64_rounds(tiles_x * tiles_y, units) * ((double)r + 0.5);
         if (cost == 0.0 || now <= cost) {
             cost = now;
             best = r;

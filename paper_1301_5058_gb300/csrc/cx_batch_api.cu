@@ -151,8 +151,8 @@ int build_work(cx_batch *B)
 
 // Tile height of a batch that has not been tuned: the default (B->rows), or
 // fewer rows so that a small batch fills the GPU: in FP32 sixteen one-warp
-// tiles of the two-stage march per SM; in FP64 the height r with the least
-// ceil(tiles / FP64 units) (r + 1/2), as for a single grid.
+// tiles of the two-stage march per SM; in FP64 the height that a single grid
+// would take.
 int auto_rows(const cx_batch *B)
 {
     const bool f64 = B->prec == CX_PREC_F64;
@@ -169,7 +169,7 @@ int auto_rows(const cx_batch *B)
         long long tiles = 0;
         for (const cx::TileGrid &s : B->sizes)
             tiles += (s.nx + cols - 1) / cols * ((s.ny + r - 1) / r) * s.count;
-        const double now = (double)((tiles + units - 1) / units) * ((double)r + 0.5);
+        const double now = cx::f64_rounds(tiles, units) * ((double)r + 0.5);
         if (cost == 0.0 || now <= cost) {
             cost = now;
             best = r;

@@ -225,6 +225,14 @@ inline int tile_count(int n, int size, int halo)
 }
 inline int tiles_x(int nx, const TilePlan &p) { return tile_count(nx, p.width(), p.halo_x()); }
 inline int tiles_y(int ny, const TilePlan &p) { return tile_count(ny, p.height(), p.halo_y()); }
+// How many row times of two warps sharing an FP64 unit a round-robin of
+// `blocks` one-warp blocks over `units` units takes per row (cx_api.cu,
+// auto_tile_rows_f64).
+inline double f64_rounds(long long blocks, long long units)
+{
+    const long long q = (blocks + units - 1) / units;
+    return q == 1 ? 1.4 : (double)q;
+}
 struct TileGrid {
     int nx, ny, count;  // `count` grids of this size
 };
