@@ -305,10 +305,11 @@ int cx_batch_set_stream(cx_batch *b, void *stream);
 /* Performance knobs, none of which changes any result bit:
  *   tile_rows   rows per tile of the step kernel (1..4096; the tiles of
  *               both depths; default 128 for FP32 batches, which take two
- *               stages per pass, 32 for FP64 ones).  A batch whose knobs and
- *               depth were never set chooses for itself, as a single grid
- *               does: fewer rows where it would leave the GPU idle, or
- *               several steps per pass on register tiles;
+ *               stages per pass, 32 for FP64 ones).  With the height,
+ *               the groups, the resident mode and the depth all at their
+ *               defaults the batch chooses for itself, as a single grid does:
+ *               fewer rows where it would leave the GPU idle, or several
+ *               steps per pass on register tiles;
  *   graph_steps steps captured per CUDA graph and replayed (0: plain
  *               launches; rounded up to even for Euler; default 64);
  *   group_bytes if > 0, instances are cut into consecutive groups whose

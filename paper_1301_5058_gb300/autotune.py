@@ -110,8 +110,10 @@ def tune_batch(batch: "cx.Batch", steps: int = 128, reps: int = 3, candidates=No
 
 
 def tune_single(sim: "cx.Sim", steps: int = 20, reps: int = 3, use_cache: bool = True):
-    """Pick the temporal blocking depth and tile height of a single grid;
-    applies the winner and returns ((time_block, rows), timings)."""
+    """Pick the temporal blocking depth and tile height of a single grid's row
+    marches; applies the winner and returns ((time_block, rows), timings).  A
+    grid of up to about 2500^2 cells is faster left alone: without a depth and
+    a height of its own it runs on register tiles (cx_set_tile_rows)."""
     import torch
     key = f"single/p{sim.params.precision}/s{sim.params.scheme}/n{sim.params.noise_mode}/" \
           f"{sim.grid.nx}x{sim.grid.ny}"

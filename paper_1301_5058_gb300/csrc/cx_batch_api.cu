@@ -67,7 +67,7 @@ struct cx_batch {
     std::vector<int> work2_begin;
     int rows = 32;                  // tile height set, or reported as the default
     int march_rows = 32;            // tile height in effect
-    bool tuned = false;             // heights or depth were set: the marches run as told
+    bool tuned = false;             // a knob of the marches is off its default: they run as told
     int num_sms = 1;
     std::vector<cx::TileGrid> sizes;  // the instances' distinct sizes
     int64_t plan_for = 0;           // steps that `plan` was made for (0: none yet)
@@ -176,6 +176,32 @@ int auto_rows(const cx_batch *B)
         }
     }
     return (int)best;
+}
+
+void build_groups(cx_batch *B);
+
+// Whether the knobs choose a march: the height, the depth, the groups or the
+// resident mode differ from the defaults.
+bool is_tuned(const cx_batch *B)
+{
+    const bool f32 = B->prec == CX_PREC_F32;
+    return B->rows != (f32 ? 128 : 32) || B->time_block != (f32 ? 2 : 1) || B->group_bytes > 0 ||
+           B->resident_steps > 0;
+}
+
+// After a knob was set: the height in effect, and the marches' work lists.
+int apply_tuning(cx_batch *B)
+{
+    B->tuned = is_tuned(B);
+    B->plan_for = 0;
+    const int rows = B->tuned ? B->rows : auto_rows(B);
+    if (rows != B->march_rows) {
+        B->march_rows = rows;
+        const int rc = build_work(B);
+        if (rc) return rc;
+    }
+    build_groups(B);
+    return CX_OK;
 }
 
 // Whether runs of `steps` steps take several steps per pass, as a single grid
@@ -556,18 +582,11 @@ int cx_batch_set_tuning(cx_batch *B, int32_t tile_rows, int32_t graph_steps, int
                                          "resident_steps 0..1000000");
     BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before retuning");
     drop_graphs(B);
-    const bool new_rows = tile_rows != B->march_rows;
-    B->rows = B->march_rows = tile_rows;
-    B->tuned = true;
+    B->rows = tile_rows;
     B->graph_steps = (B->scheme == CX_SCHEME_EULER && (graph_steps & 1)) ? graph_steps + 1 : graph_steps;
     B->group_bytes = group_bytes;
     B->resident_steps = resident_steps;
-    if (new_rows) {
-        rc = build_work(B);
-        if (rc) return rc;
-    }
-    build_groups(B);
-    return CX_OK;
+    return apply_tuning(B);
 }
 
 int cx_batch_get_tuning(cx_batch *B, int32_t *tile_rows, int32_t *graph_steps, int64_t *group_bytes,
@@ -591,8 +610,7 @@ int cx_batch_set_time_block(cx_batch *B, int32_t stages)
     BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before retuning");
     drop_graphs(B);
     B->time_block = stages;
-    B->tuned = true;
-    return CX_OK;
+    return apply_tuning(B);
 }
 
 int cx_batch_get_time_block(cx_batch *B, int32_t *stages)
