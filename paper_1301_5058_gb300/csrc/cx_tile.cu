@@ -34,6 +34,7 @@ struct Shape {
 };
 const Shape kShapes[] = {{16, 2, 128, 0.200}, {16, 2, 256, 0.200}, {16, 2, 512, 0.200},
                          {16, 4, 128, 0.185}, {16, 4, 256, 0.185}, {16, 4, 512, 0.185},
+                         {16, 6, 256, 0.175}, {16, 6, 512, 0.175},
                          {32, 6, 256, 0.175}, {32, 6, 512, 0.175}};
 const int kSteps[] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16, 32, 64, 128, 256, 512, 1024};
 

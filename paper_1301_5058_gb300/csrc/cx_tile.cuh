@@ -28,9 +28,11 @@
 // 78 %.  Euler, static sigma, us per step, marches -> tiles: 64^2 1.5 -> 0.67,
 // 256^2 2.7 -> 0.74, 512^2 3.1 -> 1.2, 1024^2 4.5 -> 2.8, 2048^2 10.1 -> 9.0;
 // Heun with per-step sigma 256^2 4.4 -> 2.1, 1024^2 19.1 -> 8.3, 2048^2
-// 37.1 -> 25.0; 96 instances of 256^2 38 -> 14.6.  Three shapes: 2 rows per
+// 37.1 -> 25.0; 96 instances of 256^2 38 -> 14.6.  Four shapes: 2 rows per
 // thread make the smallest tiles (most SMs at work), 4 and 6 rows waste less on
-// y-faces that two threads both evaluate (a share of 1/(2 R)).  A static
+// y-faces that two threads both evaluate (a share of 1/(2 R)); 6 rows of 64
+// columns stand beside those of 128 because a tall tile fits some grids better
+// (96 instances of 256^2 14.6 -> 13.4 us per step, 1501 x 1037 5.0 -> 4.7).  A static
 // sigma's face sums are kept in shared memory from stage to stage (3-5 %).
 #pragma once
 

@@ -102,6 +102,7 @@ cudaError_t launch_shape(const TileLaunch &a, const TilePlan &p, cudaStream_t st
 {
     if (p.lx == 16 && p.r == 2) return launch_v<LAW, MOB, NOISE, HEUN, 16, 2>(a, p, st);
     if (p.lx == 16 && p.r == 4) return launch_v<LAW, MOB, NOISE, HEUN, 16, 4>(a, p, st);
+    if (p.lx == 16 && p.r == 6) return launch_v<LAW, MOB, NOISE, HEUN, 16, 6>(a, p, st);
     if (p.lx == 32 && p.r == 6) return launch_v<LAW, MOB, NOISE, HEUN, 32, 6>(a, p, st);
     return cudaErrorInvalidValue;
 }
