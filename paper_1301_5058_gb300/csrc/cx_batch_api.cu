@@ -149,20 +149,28 @@ int build_work(cx_batch *B)
     return CX_OK;
 }
 
-// Tile height of a batch that has not been tuned: the default (B->rows), or
-// fewer rows so that a small batch fills the GPU: in FP32 sixteen one-warp
-// tiles of the two-stage march per SM; in FP64 the height that a single grid
-// would take.
+// Tile height of a batch that has not been tuned, in place of the default
+// (B->rows).  FP32 (two-stage march, 16 one-warp tiles per SM at a time): the
+// least height at which one round of tiles covers the batch if that is below
+// 72, else 64 rows: a round that is barely exceeded costs nearly two (16
+// instances of 1024^2: 60 rows, 1.07 rounds, 44.0 us per step; 64 rows, 0.95,
+// 36.9), and from there on 64 rows fill the rounds better than 128 (24
+// instances of 512^2 .. 2048^2 98.6 -> 87.7 us per step, 128 of them 431 -> 417,
+// 64 of 1024^2 133 -> 125).  FP64: the height that a single grid would take.
 int auto_rows(const cx_batch *B)
 {
-    const bool f64 = B->prec == CX_PREC_F64;
-    const long long cols = f64 ? tile_cols(B->prec) : kFusedTileCols, units = 4LL * B->num_sms;
-    long long columns = 0;  // tile columns x rows of all instances
-    for (const cx_grid &g : B->g) columns += (g.nx + cols - 1) / cols * g.ny;
-    if (!f64) {
-        const long long r = columns / (4 * units);
-        return (int)(r < 8 ? 8 : r < B->rows ? r : B->rows);
+    if (B->prec == CX_PREC_F32) {
+        const long long slots = 16LL * B->num_sms;
+        for (int r = 8; r < 72; ++r) {
+            long long tiles = 0;
+            for (const cx::TileGrid &s : B->sizes)
+                tiles += (long long)s.count * ((s.nx + kFusedTileCols - 1) / kFusedTileCols) *
+                         ((s.ny + r - 1) / r);
+            if (tiles <= slots) return r;
+        }
+        return 64;
     }
+    const long long cols = tile_cols(B->prec), units = 4LL * B->num_sms;
     long long best = 1;
     double cost = 0.0;
     for (long long r = 1; r <= B->rows; ++r) {
