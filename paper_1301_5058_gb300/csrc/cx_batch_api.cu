@@ -34,6 +34,7 @@ int bcuda(cudaError_t e, const char *what)
 int tile_cols(int prec) { return prec == CX_PREC_F64 ? 128 : 512; }
 constexpr int kFusedTileCols = 120;  // written columns per (one-warp) tile of the two-stage march
 constexpr int kDiagBlocksPerInst = 64;
+constexpr size_t kMaxTileWork = 32;  // tile lists kept (one per pass length and shape)
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -102,6 +103,13 @@ void drop_graphs(cx_batch *B)
     }
 }
 
+void free_tiles(cx_batch *B)
+{
+    for (TileWork &t : B->tile_work)
+        if (t.d) cudaFree(t.d);
+    B->tile_work.clear();
+}
+
 void free_batch(cx_batch *B)
 {
     if (!B) return;
@@ -111,8 +119,7 @@ void free_batch(cx_batch *B)
     if (B->d_inst) cudaFree(B->d_inst);
     if (B->d_work) cudaFree(B->d_work);
     if (B->d_work2) cudaFree(B->d_work2);
-    for (TileWork &t : B->tile_work)
-        if (t.d) cudaFree(t.d);
+    free_tiles(B);
     if (B->d_part) cudaFree(B->d_part);
     if (B->h_res) cudaFreeHost(B->h_res);
     if (B->d_barrier) cudaFree(B->d_barrier);
@@ -645,6 +652,12 @@ int cx_batch_step(cx_batch *B, int64_t n_steps)
         drop_graphs(B);
     }
     if (B->tiles) {
+        if (B->tile_work.size() > kMaxTileWork) {
+            // calls of many different lengths: start over rather than keep all
+            BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before new tile lists");
+            drop_graphs(B);
+            free_tiles(B);
+        }
         rc = whole ? build_tiles(B, B->graph_steps) : CX_OK;
         if (rc == CX_OK) rc = build_tiles(B, whole ? n_steps % B->graph_steps : n_steps);
         if (rc) return rc;

@@ -80,3 +80,35 @@ def test_untuned_batch_is_single_marches_bitwise(cx, kw, sizes):
             sim.step(64 + 27 + 5 + 64)
             assert np.array_equal(b, sim.field(cx.CX_FIELD_B, dtype))
             assert np.array_equal(n, sim.field(cx.CX_FIELD_N, dtype))
+
+
+@pytest.mark.parametrize("nx,ny,prec", [(200, 130, 1), (300, 1, 0), (96, 80, 0)])
+def test_steps_captured_in_a_graph(cx, nx, ny, prec):
+    # the passes of a step call are launched as dependents of one another;
+    # captured and replayed they give what the call itself gives
+    torch = pytest.importorskip("torch")
+    dtype = np.float32 if prec else np.float64
+    kw = dict(BASE, precision=prec)
+    with cx.Sim(nx, ny, 1.0, seed=5, **kw) as sim, cx.Sim(nx, ny, 1.0, seed=5, **kw) as ref:
+        stream = torch.cuda.Stream()
+        cx.cx_set_stream(sim.h, stream.cuda_stream)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            sim.step(23)
+        graph.replay()
+        torch.cuda.synchronize()
+        ref.step(23)
+        for which in (cx.CX_FIELD_B, cx.CX_FIELD_N):
+            assert np.array_equal(sim.field(which, dtype), ref.field(which, dtype))
+
+
+def test_tall_grids_stay_within_the_launch(cx):
+    # as many tile rows as a launch may have: the choice of tiles respects it
+    with cx.Sim(1, 2_000_000, 1.0, seed=1, **BASE) as sim, \
+            cx.Sim(1, 2_000_000, 1.0, seed=1, **BASE) as ref:
+        cx.cx_set_time_block(ref.h, 2)
+        cx.cx_set_tile_rows(ref.h, 64)
+        sim.step(6)
+        ref.step(6)
+        assert np.array_equal(sim.field(cx.CX_FIELD_B, np.float32), ref.field(cx.CX_FIELD_B, np.float32))
