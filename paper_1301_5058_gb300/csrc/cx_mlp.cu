@@ -44,7 +44,7 @@
 // a quarter of H1 and writes it into the A operand of all four (distributed
 // shared memory), and the four partial sums of Y meet in the same way.  With
 // the launches overlapped (launch_pass), a training step of 8 members x 256
-// rows takes 38 us; one CTA per 128 x 256 tile took 89.
+// rows takes 35 us; one CTA per 128 x 256 tile took 89.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>
@@ -741,19 +741,18 @@ __global__ void __launch_bounds__(kSumCols *kSumRows)
     for (int a = 0; a < 8; ++a) part[ty][a][tx] = acc[a];
     __syncthreads();
     float *G = v.G + (long long)e * NPARAM;
-    if (ty == 0) {
-        float s[8];
+    if (threadIdx.x < 8 * kSumCols) {
+        // one thread per sum and column (the 16 threads of one thread row took
+        // all eight sums one after the other)
+        const int k = threadIdx.x / kSumCols;
+        float sum = part[0][k][tx];
 #pragma unroll
-        for (int a = 0; a < 8; ++a) {
-            s[a] = part[0][a][tx];
-            for (int y = 1; y < kSumRows; ++y) s[a] += part[y][a][tx];
-        }
-        G[OFF_W3 + j] = s[0];
-        G[OFF_W3 + H + j] = s[1];
-        G[OFF_B2 + j] = s[2];
-#pragma unroll
-        for (int k = 0; k < NI; ++k) G[OFF_W1 + j * NI + k] = s[3 + k];
-        G[OFF_B1 + j] = s[7];
+        for (int y = 1; y < kSumRows; ++y) sum += part[y][k][tx];
+        float *dst = k < NO ? G + OFF_W3 + k * H + j
+                     : k == 2 ? G + OFF_B2 + j
+                     : k < 7  ? G + OFF_W1 + j * NI + (k - 3)
+                              : G + OFF_B1 + j;
+        *dst = sum;
     }
     if (blockIdx.x == 0) {
         const int tid = ty * kSumCols + tx, nth = kSumRows * kSumCols;
@@ -787,29 +786,48 @@ __global__ void __launch_bounds__(kSumCols *kSumRows)
     }
 }
 
-// Adam (Kingma & Ba, 2015) on the FP32 master parameters of every member;
-// the threads of W2 entries also write the bf16 copies of W2 and W2^T.
-__global__ void adam_kernel(float *P, const float *G, float *M, float *V, __nv_bfloat16 *W2b,
-                            __nv_bfloat16 *W2T, long long n, float lr, float b1, float b2, float eps,
-                            float c1, float c2)
+// Adam (Kingma & Ba, 2015) on the FP32 master parameters of member blockIdx.y.
+// The first blocks take 32 x 32 tiles of W2 and also write its bf16 copies, the
+// transposed one through shared memory (written straight, its 2-byte stores
+// lie 512 bytes apart; with column_sums' last additions spread over 128
+// threads 37.7 -> 35.2 us per step); the others take the rest of the parameters.
+constexpr int kAdamTile = 32, kAdamTiles = (H / kAdamTile) * (H / kAdamTile);
+constexpr int kAdamRest = (NPARAM - H * H + 255) / 256;
+__global__ void __launch_bounds__(256)
+    adam_kernel(float *P, const float *G, float *M, float *V, __nv_bfloat16 *W2b, __nv_bfloat16 *W2T,
+                float lr, float b1, float b2, float eps, float c1, float c2)
 {
+    __shared__ __nv_bfloat16 tile[kAdamTile][kAdamTile + 2];
     cx::pass_wait();
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float g = G[i];
-    const float m = b1 * M[i] + (1.f - b1) * g;
-    const float vv = b2 * V[i] + (1.f - b2) * g * g;
-    M[i] = m;
-    V[i] = vv;
-    const float p = P[i] - lr * (m / c1) / (sqrtf(vv / c2) + eps);
-    P[i] = p;
-    const long long e = i / NPARAM;
-    const int o = (int)(i - e * NPARAM) - OFF_W2;
-    if (o >= 0 && o < H * H) {
-        const __nv_bfloat16 w = __float2bfloat16_rn(p);
-        W2b[e * H * H + o] = w;
-        W2T[e * H * H + (o % H) * H + o / H] = w;
+    const long long e = blockIdx.y, base = e * NPARAM;
+    auto update = [&](long long i) -> float {
+        const float g = G[i];
+        const float m = b1 * M[i] + (1.f - b1) * g;
+        const float vv = b2 * V[i] + (1.f - b2) * g * g;
+        M[i] = m;
+        V[i] = vv;
+        const float p = P[i] - lr * (m / c1) / (sqrtf(vv / c2) + eps);
+        P[i] = p;
+        return p;
+    };
+    if (blockIdx.x >= kAdamTiles) {
+        const int q = (blockIdx.x - kAdamTiles) * 256 + threadIdx.x;
+        if (q < NPARAM - H * H) update(base + (q < OFF_W2 ? q : q + H * H));
+        return;
     }
+    const int r0 = blockIdx.x / (H / kAdamTile) * kAdamTile, k0 = blockIdx.x % (H / kAdamTile) * kAdamTile;
+    const int x = threadIdx.x % kAdamTile, y0 = threadIdx.x / kAdamTile;
+#pragma unroll
+    for (int y = y0; y < kAdamTile; y += 256 / kAdamTile) {
+        const int o = (r0 + y) * H + k0 + x;
+        const __nv_bfloat16 w = __float2bfloat16_rn(update(base + OFF_W2 + o));
+        W2b[e * H * H + o] = w;
+        tile[y][x] = w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int y = y0; y < kAdamTile; y += 256 / kAdamTile)
+        W2T[e * H * H + (k0 + y) * H + r0 + x] = tile[x][y];
 }
 
 // bf16 copies of every member's W2 (row-major) and W2^T.
@@ -1106,7 +1124,6 @@ int cx_mlp_train(cx_mlp *m, const float *x, const float *t, int32_t n, int32_t b
     }
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const int nbatches = n / batch;
-    const long long np = E * NPARAM;
     for (int s = 0; s < steps; ++s) {
         const long long first = (long long)(s % nbatches) * batch;  // cyclic minibatches
         MX_CUDA(run_pass(m, m->dataX + first * NI, (long long)n * NI, m->dataT + first * NO,
@@ -1114,8 +1131,8 @@ int cx_mlp_train(cx_mlp *m, const float *x, const float *t, int32_t n, int32_t b
                 "training pass");
         m->adam_t += 1;
         const float c1 = 1.f - powf(b1, (float)m->adam_t), c2 = 1.f - powf(b2, (float)m->adam_t);
-        MX_CUDA(cx::launch_pass(adam_kernel, (unsigned)((np + 255) / 256), 256, 0, m->st, m->P, m->G, m->M,
-                                m->V, m->W2b, m->W2T, np, lr, b1, b2, eps, c1, c2),
+        MX_CUDA(cx::launch_pass(adam_kernel, dim3(kAdamTiles + kAdamRest, (unsigned)E), 256, 0, m->st,
+                                m->P, m->G, m->M, m->V, m->W2b, m->W2T, lr, b1, b2, eps, c1, c2),
                 "optimiser launch");
     }
     if (loss_out && steps > 0)
