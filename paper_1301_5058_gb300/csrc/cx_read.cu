@@ -61,19 +61,19 @@ cudaError_t launch_read(const void *a, void *dst, int nx, int ny, long long pitc
     return launch_pass(kern, grid, 256, 0, st, (const T *)a, (D *)dst, nx, ny, pitch);
 }
 
-using PointerAttributeFn = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+using PointerAttributesFn = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
 
-PointerAttributeFn pointer_attribute()
+PointerAttributesFn pointer_attributes()
 {
     static std::once_flag once;
-    static PointerAttributeFn fn = nullptr;
+    static PointerAttributesFn fn = nullptr;
     std::call_once(once, [] {
         void *f = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) ==
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) ==
                 cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            fn = (PointerAttributeFn)f;
+            fn = (PointerAttributesFn)f;
         cudaGetLastError();
     });
     return fn;
@@ -83,22 +83,20 @@ PointerAttributeFn pointer_attribute()
 
 void *pinned_view(void *host, size_t bytes)
 {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+    const PointerAttributesFn get = pointer_attributes();
+    if (!get) return nullptr;
+    // one query: memory that CUDA does not know comes back as type 0
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned type = 0;
+    CUdeviceptr p = 0, start = 0;
+    size_t size = 0;
+    void *values[] = {&type, &p, &start, &size};
+    if (get(4, what, values, (CUdeviceptr)host) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || !p) return nullptr;
     // the whole array has to lie in the pinned allocation (one that does not is
     // left to the copies, which refuse it)
-    const PointerAttributeFn get = pointer_attribute();
-    CUdeviceptr start = 0;
-    size_t size = 0;
-    const CUdeviceptr p = (CUdeviceptr)at.devicePointer;
-    if (!get || get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, p) != CUDA_SUCCESS ||
-        get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, p) != CUDA_SUCCESS)
-        return nullptr;
-    return p >= start && p + bytes <= start + size ? at.devicePointer : nullptr;
+    return p >= start && p + bytes <= start + size ? (void *)p : nullptr;
 }
 
 cudaError_t launch_read_field(int prec, const void *field, int nx, int ny, long long pitch, void *dst,
