@@ -75,9 +75,13 @@ struct Coef {
     double cN;    // dt
 };
 
-// The FP64 receptor law's scale without chemotaxis: the weight is then 2^-1002,
-// below the rounding of any flux (and the square of the denominator is finite).
-constexpr double kNoChemoF64 = 0x1p500;
+// The FP64 receptor law's largest scale (chi0 = 0, and chi0 below about 1e-39):
+// the weight is then at most 2^-128, far below the rounding of any flux, and the
+// square of the denominator, 2^128 (2 + n_L + n_R)^2, is finite up to
+// n_L + n_R = 2^447.  A larger scale loses that range for nothing (2^500
+// overflowed from n_L + n_R = 4094 on, and the reciprocal's correction made
+// 0 inf of it).
+constexpr double kNoChemoF64 = 0x1p64;
 
 struct Sigma {  // how sigma is obtained
     int per_step;     // 0: read the sigma array; 1: regenerate from Philox every step
