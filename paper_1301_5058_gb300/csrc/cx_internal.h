@@ -221,11 +221,12 @@ struct TilePlan {
     int halo_y() const { return stages(); }
 };
 // Tiles along a side of n cells; the first and the last lie against the walls
-// and need no halo there.
+// and need no halo there.  0: tiles of this size keep no cell of such a side.
 inline int tile_count(int n, int size, int halo)
 {
     const int step = size - 2 * halo;
-    return n <= size ? 1 : 1 + (n - size + step - 1) / step;
+    if (n <= size) return 1;
+    return step <= 0 ? 0 : 1 + (n - size + step - 1) / step;
 }
 inline int tiles_x(int nx, const TilePlan &p) { return tile_count(nx, p.width(), p.halo_x()); }
 inline int tiles_y(int ny, const TilePlan &p) { return tile_count(ny, p.height(), p.halo_y()); }

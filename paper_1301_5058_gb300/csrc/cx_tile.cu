@@ -67,9 +67,9 @@ double plan_tiles(const TileGrid *grids, int count, int sms, bool heun, bool per
             for (int i = 0; i < count && tiles >= 0.0; ++i) {
                 // tiles that keep less than a quarter of their cells do not pay
                 // (and a single grid's tile rows have to fit its launch)
-                const bool fits = tiles_y(grids[i].ny, p) <= 65535 &&
-                                  (grids[i].nx <= p.width() || 2 * (p.width() - 2 * p.halo_x()) >= p.width()) &&
-                                  (grids[i].ny <= p.height() || 2 * (p.height() - 2 * p.halo_y()) >= p.height());
+                const bool fits = (grids[i].nx <= p.width() || 2 * (p.width() - 2 * p.halo_x()) >= p.width()) &&
+                                  (grids[i].ny <= p.height() || 2 * (p.height() - 2 * p.halo_y()) >= p.height()) &&
+                                  tiles_y(grids[i].ny, p) <= 65535;
                 if (fits)
                     tiles += (double)grids[i].count * tiles_x(grids[i].nx, p) * tiles_y(grids[i].ny, p);
                 else
