@@ -645,7 +645,7 @@ int cx_get_field(cx_ctx *c, int32_t which, void *host, int32_t dtype, size_t cou
     if (which == CX_FIELD_SIGMA && c->p.noise_mode == CX_NOISE_PER_STEP)
         CX_CUDA(fill_sigma(c, c->step), "sigma regeneration");
     void *f = field_ptr(c, which);
-    if (void *view = cx::pinned_view(host, count * (dtype == CX_F64 ? 8 : 4))) {
+    if (void *view = cx::pinned_view(host, count, dtype == CX_F64 ? 8 : 4)) {
         CX_CUDA(cx::launch_read_field(c->prec, f, c->g.nx, c->g.ny, c->pitch, view, dtype, c->stream),
                 "field read");
         CX_CUDA(cudaStreamSynchronize(c->stream), "field read synchronize");

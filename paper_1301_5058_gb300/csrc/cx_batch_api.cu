@@ -782,7 +782,7 @@ int cx_batch_get_field(cx_batch *B, int32_t index, int32_t which, void *host, in
     if (!host) return bfail(CX_ERR_INVALID_ARG, "host must not be NULL");
     const int sd = B->prec == CX_PREC_F64 ? CX_F64 : CX_F32;
     const size_t row = (size_t)B->g[index].nx * B->elem;
-    if (void *view = cx::pinned_view(host, count * (dtype == CX_F64 ? 8 : 4))) {
+    if (void *view = cx::pinned_view(host, count, dtype == CX_F64 ? 8 : 4)) {
         BX_CUDA(cx::launch_read_field(B->prec, batch_field(B, index, which), B->g[index].nx,
                                       B->g[index].ny, B->pitch[index], view, dtype, B->stream),
                 "field read");

@@ -137,9 +137,10 @@ __host__ __device__ __forceinline__ long long pair_col(long long i)
 // natural in-row order and the pair order (either way).
 cudaError_t launch_pair_order(int prec, void *a, int nx, int ny, long long pitch, cudaStream_t st);
 
-// The address under which a kernel may write the `bytes` bytes at `host`, or
-// nullptr unless all of them are pinned (cx_read.cu).
-void *pinned_view(void *host, size_t bytes);
+// The address under which a kernel may write the `count` elements of `elem`
+// bytes at `host`, or nullptr unless all of them are pinned and aligned to
+// their size (cx_read.cu).
+void *pinned_view(void *host, size_t count, size_t elem);
 // A field in pair order -> packed rows of nx elements in natural order and of
 // type `dtype` (CX_F64 / CX_F32) at `dst`, device or pinned host memory.
 cudaError_t launch_read_field(int prec, const void *field, int nx, int ny, long long pitch, void *dst,

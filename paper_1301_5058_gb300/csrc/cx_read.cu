@@ -81,8 +81,11 @@ PointerAttributesFn pointer_attributes()
 
 }  // namespace
 
-void *pinned_view(void *host, size_t bytes)
+void *pinned_view(void *host, size_t count, size_t elem)
 {
+    // a kernel stores whole elements: an array behind an odd-sized header goes
+    // through the copies
+    if ((uintptr_t)host % elem) return nullptr;
     const PointerAttributesFn get = pointer_attributes();
     if (!get) return nullptr;
     // one query: memory that CUDA does not know comes back as type 0
@@ -96,7 +99,7 @@ void *pinned_view(void *host, size_t bytes)
     if (type != CU_MEMORYTYPE_HOST || !p) return nullptr;
     // the whole array has to lie in the pinned allocation (one that does not is
     // left to the copies, which refuse it)
-    return p >= start && p + bytes <= start + size ? (void *)p : nullptr;
+    return p % elem == 0 && p >= start && p + count * elem <= start + size ? (void *)p : nullptr;
 }
 
 cudaError_t launch_read_field(int prec, const void *field, int nx, int ny, long long pitch, void *dst,
