@@ -651,27 +651,23 @@ int cx_get_field(cx_ctx *c, int32_t which, void *host, int32_t dtype, size_t cou
         CX_CUDA(cudaStreamSynchronize(c->stream), "field read synchronize");
         return CX_OK;
     }
-    // the array in natural in-row order for the copy, and back afterwards
-    CX_CUDA(cx::launch_pair_order(c->prec, f, c->g.nx, c->g.ny, c->pitch, c->stream), "reorder");
-    if (dtype == state_dtype) {
-        CX_CUDA(copy_rows(host, row, f, (size_t)c->pitch * c->elem, row, c->g.ny,
-                          cudaMemcpyDeviceToHost, c->stream),
-                "field copy to host");
-        CX_CUDA(cx::launch_pair_order(c->prec, f, c->g.nx, c->g.ny, c->pitch, c->stream), "reorder");
-        CX_CUDA(cudaStreamSynchronize(c->stream), "field copy synchronize");
-        return CX_OK;
-    }
     // precision change: copy in the state type, widen or narrow on the host
     std::vector<unsigned char> tmp;
-    try { tmp.resize(count * c->elem); } catch (...) {
-        cx::launch_pair_order(c->prec, f, c->g.nx, c->g.ny, c->pitch, c->stream);
-        return fail(CX_ERR_OOM, "host staging");
+    void *dst = host;
+    if (dtype != state_dtype) {
+        try { tmp.resize(count * c->elem); } catch (...) { return fail(CX_ERR_OOM, "host staging"); }
+        dst = tmp.data();
     }
-    CX_CUDA(copy_rows(tmp.data(), row, f, (size_t)c->pitch * c->elem, row, c->g.ny,
-                      cudaMemcpyDeviceToHost, c->stream),
-            "field copy to host");
+    // the array in natural in-row order for the copy, and back afterwards, also
+    // when the copy was refused (an array that is pinned in part)
     CX_CUDA(cx::launch_pair_order(c->prec, f, c->g.nx, c->g.ny, c->pitch, c->stream), "reorder");
+    const cudaError_t copied = copy_rows(dst, row, f, (size_t)c->pitch * c->elem, row, c->g.ny,
+                                         cudaMemcpyDeviceToHost, c->stream);
+    if (copied != cudaSuccess) cudaGetLastError();  // reported below, not by the launch
+    CX_CUDA(cx::launch_pair_order(c->prec, f, c->g.nx, c->g.ny, c->pitch, c->stream), "reorder");
+    CX_CUDA(copied, "field copy to host");
     CX_CUDA(cudaStreamSynchronize(c->stream), "field copy synchronize");
+    if (dtype == state_dtype) return CX_OK;
     if (state_dtype == CX_F32) {
         const float *s = (const float *)tmp.data();
         double *d = (double *)host;

@@ -796,14 +796,17 @@ int cx_batch_get_field(cx_batch *B, int32_t index, int32_t which, void *host, in
         dst = tmp.data();
     }
     BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before field read");
-    // the array in natural in-row order for the copy, and back to pair order
+    // the array in natural in-row order for the copy, and back to pair order, also
+    // when the copy was refused (an array that is pinned in part)
     void *f = batch_field(B, index, which);
     const cx_grid &g = B->g[index];
     BX_CUDA(cx::launch_pair_order(B->prec, f, g.nx, g.ny, B->pitch[index], B->stream), "reorder");
-    BX_CUDA(cudaMemcpy2DAsync(dst, row, f, (size_t)B->pitch[index] * B->elem,
-                              row, B->g[index].ny, cudaMemcpyDeviceToHost, B->stream),
-            "field copy to host");
+    const cudaError_t copied =
+        cudaMemcpy2DAsync(dst, row, f, (size_t)B->pitch[index] * B->elem, row, B->g[index].ny,
+                          cudaMemcpyDeviceToHost, B->stream);
+    if (copied != cudaSuccess) cudaGetLastError();  // reported below, not by the launch
     BX_CUDA(cx::launch_pair_order(B->prec, f, g.nx, g.ny, B->pitch[index], B->stream), "reorder");
+    BX_CUDA(copied, "field copy to host");
     BX_CUDA(cudaStreamSynchronize(B->stream), "field copy synchronize");
     if (dtype != sd) {
         if (sd == CX_F32)

@@ -35,3 +35,42 @@ def test_pinned_array_not_aligned_to_its_elements(cx, prec, dtype, offset):
                 host[offset:offset + size] = 0
                 assert np.array_equal(get(which), ref(which, dtype))
         assert np.all(host[:offset] == 7) and np.all(host[offset + size:] == 7)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_refused_copy_leaves_the_state_as_it_was(cx, prec):
+    # the runtime refuses a copy into an array that is pinned only in part; the
+    # field has to be back in the library's order all the same
+    torch = pytest.importorskip("torch")
+    dtype = np.float32 if prec else np.float64
+    nx, ny = 128, 256
+    kw = dict(KW, precision=prec)
+    page = 65536  # a whole number of pages on any host
+    with cx.Sim(nx, ny, 1.0, seed=3, **kw) as sim, \
+            cx.Batch([dict(nx=nx, ny=ny, dx=1.0, seed=3, **kw)]) as bt:
+        whole = np.zeros(8 * page, np.uint8)
+        first = -whole.ctypes.data % page
+        out = whole[first:first + nx * ny * np.dtype(dtype).itemsize].view(dtype).reshape(ny, nx)
+        assert out.nbytes > page
+        rt = torch.cuda.cudart()
+        for get, read, step in (
+                (lambda: cx.cx_get_field(sim.h, cx.CX_FIELD_B, out),
+                 lambda: sim.field(cx.CX_FIELD_B, dtype), sim.step),
+                (lambda: cx.cx_batch_get_field(bt.h, 0, cx.CX_FIELD_B, out),
+                 lambda: bt.field(0, cx.CX_FIELD_B, dtype), bt.step)):
+            want = read()
+            assert int(rt.cudaHostRegister(out.ctypes.data, page, 0)) == 0
+            try:
+                try:
+                    get()
+                    refused = False
+                except cx.CxError:
+                    refused = True
+            finally:
+                assert int(rt.cudaHostUnregister(out.ctypes.data)) == 0
+            assert refused or np.array_equal(out, want)
+            assert np.array_equal(read(), want)
+            step(1)
+        assert refused  # on this runtime
+        for which in (cx.CX_FIELD_B, cx.CX_FIELD_N):
+            assert np.array_equal(sim.field(which, dtype), bt.field(0, which, dtype))
