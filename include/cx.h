@@ -338,7 +338,11 @@ int cx_batch_get_tuning(cx_batch *b, int32_t *tile_rows, int32_t *graph_steps, i
 int cx_batch_set_time_block(cx_batch *b, int32_t stages);
 int cx_batch_get_time_block(cx_batch *b, int32_t *stages);
 
-/* Advance every instance by n_steps >= 0 steps.  Asynchronous. */
+/* Advance every instance by n_steps >= 0 steps.  Asynchronous.  A call of fewer
+ * than graph_steps steps (any call if graph_steps is 0) is launches alone, of
+ * whatever length: it neither allocates nor waits, a caller may capture it on
+ * the batch's stream, and what was captured stays valid until the batch is
+ * tuned again or freed. */
 int cx_batch_step(cx_batch *b, int64_t n_steps);
 int cx_batch_synchronize(cx_batch *b);
 

@@ -34,16 +34,8 @@ int bcuda(cudaError_t e, const char *what)
 int tile_cols(int prec) { return prec == CX_PREC_F64 ? 128 : 512; }
 constexpr int kFusedTileCols = 120;  // written columns per (one-warp) tile of the two-stage march
 constexpr int kDiagBlocksPerInst = 64;
-constexpr size_t kMaxTileWork = 32;  // tile lists kept (one per pass length and shape)
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
-// Register tiles (cx_tile.cu) of every instance for passes of plan.steps steps.
-struct TileWork {
-    cx::TilePlan plan;
-    int4 *d = nullptr;
-    std::vector<int> begin;  // first tile of each instance (+ total)
-};
 
 }  // namespace
 
@@ -74,7 +66,7 @@ struct cx_batch {
     int64_t plan_for = 0;           // steps that `plan` was made for (0: none yet)
     bool tiles = false;             // passes run on register tiles
     cx::TilePlan plan{};
-    std::vector<TileWork> tile_work;  // by pass length
+    void *d_by_size = nullptr;      // the instance table, size by size as in `sizes`
     int graph_steps = 64;
     long long group_bytes = 0;
     int time_block = 1;             // explicit stages per pass (1 or 2)
@@ -103,13 +95,6 @@ void drop_graphs(cx_batch *B)
     }
 }
 
-void free_tiles(cx_batch *B)
-{
-    for (TileWork &t : B->tile_work)
-        if (t.d) cudaFree(t.d);
-    B->tile_work.clear();
-}
-
 void free_batch(cx_batch *B)
 {
     if (!B) return;
@@ -119,13 +104,21 @@ void free_batch(cx_batch *B)
     if (B->d_inst) cudaFree(B->d_inst);
     if (B->d_work) cudaFree(B->d_work);
     if (B->d_work2) cudaFree(B->d_work2);
-    free_tiles(B);
+    if (B->d_by_size) cudaFree(B->d_by_size);
     if (B->d_part) cudaFree(B->d_part);
     if (B->h_res) cudaFreeHost(B->h_res);
     if (B->d_barrier) cudaFree(B->d_barrier);
     if (B->d_step) cudaFree(B->d_step);
     if (B->own_stream && B->stream) cudaStreamDestroy(B->stream);
     delete B;
+}
+
+// A host table to the device, complete when the call returns: the passes, on
+// this stream, may read it before they wait for the kernels ahead of them.
+cudaError_t upload(cx_batch *B, void *dst, const void *src, size_t bytes)
+{
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, B->stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(B->stream) : e;
 }
 
 // Tile work lists for the current tile height, instance by instance: the
@@ -150,8 +143,7 @@ int build_work(cx_batch *B)
         if (d) cudaFree(d);
         d = nullptr;
         BX_CUDA(cudaMalloc((void **)&d, w.size() * sizeof(int4)), "work list allocation");
-        BX_CUDA(cudaMemcpy(d, w.data(), w.size() * sizeof(int4), cudaMemcpyHostToDevice),
-                "work list upload");
+        BX_CUDA(upload(B, d, w.data(), w.size() * sizeof(int4)), "work list upload");
     }
     return CX_OK;
 }
@@ -255,46 +247,6 @@ int tile_pass_steps(const cx_batch *B, int64_t left)
     return (int)((left + passes - 1) / passes);
 }
 
-// The tiles for passes of the plan's shape and `steps` steps, built once.
-TileWork *find_tiles(cx_batch *B, int steps)
-{
-    for (TileWork &t : B->tile_work)
-        if (t.plan.steps == steps && t.plan.lx == B->plan.lx && t.plan.r == B->plan.r &&
-            t.plan.threads == B->plan.threads)
-            return &t;
-    return nullptr;
-}
-
-// Builds what the passes of a run of `left` steps need (not during a capture).
-int build_tiles(cx_batch *B, int64_t left)
-{
-    while (left > 0) {
-        const int steps = tile_pass_steps(B, left);
-        left -= steps;
-        if (find_tiles(B, steps)) continue;
-        TileWork t;
-        t.plan = B->plan;
-        t.plan.steps = steps;
-        std::vector<int4> w;
-        t.begin.assign(B->count + 1, 0);
-        for (int i = 0; i < B->count; ++i) {
-            t.begin[i] = (int)w.size();
-            const int tx = cx::tiles_x(B->g[i].nx, t.plan), ty = cx::tiles_y(B->g[i].ny, t.plan);
-            for (int y = 0; y < ty; ++y)
-                for (int x = 0; x < tx; ++x) w.push_back(make_int4(i, x, y, 0));
-        }
-        t.begin[B->count] = (int)w.size();
-        BX_CUDA(cudaMalloc((void **)&t.d, w.size() * sizeof(int4)), "tile list allocation");
-        const cudaError_t e = cudaMemcpy(t.d, w.data(), w.size() * sizeof(int4), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) {
-            cudaFree(t.d);
-            return bcuda(e, "tile list upload");
-        }
-        B->tile_work.push_back(t);
-    }
-    return CX_OK;
-}
-
 // Consecutive groups of instances whose fields fit group_bytes (one group
 // with every instance when group_bytes == 0; an instance larger than the
 // budget forms a group of its own).
@@ -341,6 +293,50 @@ cudaError_t one_step(cx_batch *B, int i0, int i1, int parity, int step_off)
     return e;
 }
 
+// The runs of the batch's instances for passes of `plan`.
+void fill_runs(const cx_batch *B, const cx::TilePlan &plan, cx::TileRuns *z)
+{
+    const size_t sizes = B->sizes.size();
+    z->n = (int)std::min<size_t>(sizes, cx::kTileRuns);
+    int place = 0, first = 0;
+    for (int k = 0; k < z->n; ++k) {
+        const size_t s0 = sizes * k / z->n, s1 = sizes * (k + 1) / z->n;
+        cx::TileRun r{first, 0, place, s1 - s0 == 1 ? cx::tiles_x(B->sizes[s0].nx, plan) : 0};
+        for (size_t i = s0; i < s1; ++i) {
+            const cx::TileGrid &g = B->sizes[i];
+            r.tiles = std::max(r.tiles, cx::tiles_x(g.nx, plan) * cx::tiles_y(g.ny, plan));
+            place += g.count;
+        }
+        first += r.tiles * (place - r.place);
+        z->run[k] = r;
+    }
+    z->run[z->n] = cx::TileRun{first, 0, place, 0};
+    z->shift = 0;
+    while (first > ((long long)cx::kTileIndex << z->shift)) ++z->shift;
+    for (int i = 0, k = 0; i <= cx::kTileIndex; ++i) {
+        const long long blk = std::min<long long>(first - 1, (long long)i << z->shift);
+        while (z->run[k + 1].first <= blk) ++k;
+        z->index[i] = (unsigned short)k;
+    }
+}
+
+// One pass of `steps` steps over every instance on register tiles or strips
+// (an untuned batch has one group).
+cudaError_t tile_pass(cx_batch *B, int parity, int steps, int step_off)
+{
+    cx::TilePlan plan = B->plan;
+    plan.steps = steps;
+    cx::TileRuns runs{};
+    fill_runs(B, plan, &runs);
+    cx::TileLaunch a{};
+    a.inst = B->d_by_size;
+    a.runs = &runs;
+    a.parity = parity;
+    a.nz = pass_noise(B, step_off);
+    return B->prec == CX_PREC_F64 ? cx::launch_strip(B->law, B->mob, a, plan, B->stream)
+                                  : cx::launch_tile(B->law, B->mob, B->noise != 0, a, plan, B->stream);
+}
+
 int next_parity(const cx_batch *B, int parity) { return B->scheme == CX_SCHEME_HEUN ? parity : parity ^ 1; }
 
 // One pass over instances [i0, i1) starting at *parity, step_off steps
@@ -353,18 +349,9 @@ cudaError_t one_pass(cx_batch *B, int i0, int i1, int *parity, int64_t left, int
     const bool heun = B->scheme == CX_SCHEME_HEUN;
     if (B->tiles) {
         *steps = tile_pass_steps(B, left);
-        const TileWork *t = find_tiles(B, *steps);
-        if (!t) return cudaErrorInvalidValue;
-        cx::TileLaunch a{};
-        a.inst = B->d_inst;
-        a.work = t->d + t->begin[i0];
-        a.nwork = t->begin[i1] - t->begin[i0];
-        a.parity = *parity;
-        a.nz = pass_noise(B, step_off);
+        const cudaError_t e = tile_pass(B, *parity, *steps, step_off);
         *parity ^= 1;
-        return B->prec == CX_PREC_F64
-                   ? cx::launch_strip(B->law, B->mob, a, t->plan, B->stream)
-                   : cx::launch_tile(B->law, B->mob, B->noise != 0, a, t->plan, B->stream);
+        return e;
     }
     if (B->time_block == 2 && (heun || left >= 2)) {
         const int w0 = B->work2_begin[i0], w1 = B->work2_begin[i1];
@@ -510,7 +497,7 @@ int cx_batch_create(int32_t count, const cx_grid *grids, const cx_params *params
     if (e != cudaSuccess) { free_batch(B); return bcuda(e, "stream creation"); }
     B->own_stream = true;
     e = cudaMalloc(&B->arena, total);
-    if (e == cudaSuccess) e = cudaMemset(B->arena, 0, total);
+    if (e == cudaSuccess) e = cudaMemsetAsync(B->arena, 0, total, B->stream);
     if (e != cudaSuccess) { cudaGetLastError(); free_batch(B); return bcuda(e, "arena allocation"); }
     for (int q = 0; q < 2; ++q) {
         B->fb[q].resize(count);
@@ -534,13 +521,26 @@ int cx_batch_create(int32_t count, const cx_grid *grids, const cx_params *params
                       cx::make_coef(grids[i], params[i], B->dt[i]), cx::envelope_level(params[i]),
                       seeds[i], params[i].sigma0, params[i].noise_amp, params[i].noise_dist);
     e = cudaMalloc(&B->d_inst, B->h_inst.size());
-    if (e == cudaSuccess) e = cudaMemcpy(B->d_inst, B->h_inst.data(), B->h_inst.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(B, B->d_inst, B->h_inst.data(), B->h_inst.size());
     if (e == cudaSuccess) e = cudaMalloc((void **)&B->d_part, 8 * sizeof(double) * (size_t)count * kDiagBlocksPerInst);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&B->h_res, 8 * sizeof(double) * (size_t)count);
     if (e == cudaSuccess) e = cudaMalloc(&B->d_barrier, cx::grid_barrier_bytes());
-    if (e == cudaSuccess) e = cudaMemset(B->d_barrier, 0, cx::grid_barrier_bytes());
+    if (e == cudaSuccess) e = cudaMemsetAsync(B->d_barrier, 0, cx::grid_barrier_bytes(), B->stream);
     if (e == cudaSuccess && B->noise) e = cudaMalloc((void **)&B->d_step, sizeof(long long));
-    if (e == cudaSuccess && B->noise) e = cudaMemset(B->d_step, 0, sizeof(long long));
+    if (e == cudaSuccess && B->noise) e = cudaMemsetAsync(B->d_step, 0, sizeof(long long), B->stream);
+    // the instances by area, then by width
+    std::map<std::pair<long long, int>, std::vector<int>> sizes;
+    for (int i = 0; i < count; ++i)
+        sizes[{(long long)grids[i].nx * grids[i].ny, grids[i].nx}].push_back(i);
+    std::vector<unsigned char> by_size;
+    for (const auto &z : sizes) {
+        const cx_grid &g = grids[z.second[0]];
+        B->sizes.push_back(cx::TileGrid{g.nx, g.ny, (int)z.second.size()});
+        for (int i : z.second)
+            by_size.insert(by_size.end(), B->h_inst.begin() + isz * i, B->h_inst.begin() + isz * (i + 1));
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&B->d_by_size, by_size.size());
+    if (e == cudaSuccess) e = upload(B, B->d_by_size, by_size.data(), by_size.size());
     if (e != cudaSuccess) { cudaGetLastError(); free_batch(B); return bcuda(e, "batch tables"); }
     if (const char *s = getenv("CX_BARRIER_SPIN_LIMIT")) B->spin_limit = atoll(s);
     int dev = 0;
@@ -550,9 +550,6 @@ int cx_batch_create(int32_t count, const cx_grid *grids, const cx_params *params
         cudaGetLastError();
         B->num_sms = 1;  // only the choice of tiles uses it
     }
-    std::map<std::pair<int, int>, int> sizes;
-    for (int i = 0; i < count; ++i) sizes[{grids[i].nx, grids[i].ny}] += 1;
-    for (const auto &z : sizes) B->sizes.push_back(cx::TileGrid{z.first.first, z.first.second, z.second});
     B->march_rows = auto_rows(B);
     int rc = build_work(B);
     if (rc) { free_batch(B); return rc; }
@@ -645,23 +642,8 @@ int cx_batch_step(cx_batch *B, int64_t n_steps)
     if (n_steps < 0) return bfail(CX_ERR_INVALID_ARG, "n_steps < 0");
     if (n_steps == 0) return CX_OK;
     const bool whole = B->graph_steps > 0 && n_steps >= B->graph_steps;  // at least one graph
-    const bool was_tiles = B->tiles;
+    // (the graphs hold the plan for graph_steps, which only a knob changes)
     B->tiles = use_tiles(B, whole ? B->graph_steps : n_steps);
-    if (B->tiles != was_tiles) {
-        BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before new graphs");
-        drop_graphs(B);
-    }
-    if (B->tiles) {
-        if (B->tile_work.size() > kMaxTileWork) {
-            // calls of many different lengths: start over rather than keep all
-            BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before new tile lists");
-            drop_graphs(B);
-            free_tiles(B);
-        }
-        rc = whole ? build_tiles(B, B->graph_steps) : CX_OK;
-        if (rc == CX_OK) rc = build_tiles(B, whole ? n_steps % B->graph_steps : n_steps);
-        if (rc) return rc;
-    }
     const int ngroups = (int)B->group_first.size() - 1;
     if (B->graph_steps > 0 && (int)B->gexec[0].size() != ngroups) {
         drop_graphs(B);

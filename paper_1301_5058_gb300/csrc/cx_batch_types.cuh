@@ -41,6 +41,25 @@ __device__ __forceinline__ stencil::NoiseT<T> inst_noise(const InstDev<T> &I, ui
     return nz;
 }
 
+// What block `blk` of a pass over z works on: the instance's place in the table,
+// which of its tiles, and how many of them lie side by side (0: see TileRuns).
+struct TileAt {
+    int place, tile, across;
+};
+__device__ __forceinline__ TileAt tile_of_block(const TileRuns &z, int blk)
+{
+    const int i0 = blk >> z.shift;
+    int k = z.index[i0], last = z.index[i0 + 1];
+    while (k < last) {
+        const int mid = (k + last + 1) / 2;
+        if (blk < z.run[mid].first) last = mid - 1;
+        else k = mid;
+    }
+    const TileRun r = z.run[k];
+    const int t = blk - r.first, i = t / r.tiles;
+    return TileAt{r.place + i, t - i * r.tiles, r.across};
+}
+
 // State of the resident kernel's grid-wide barrier (cx_batch_kernels.cuh).
 struct GridBarrier {
     unsigned count, gen;

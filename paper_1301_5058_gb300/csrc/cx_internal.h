@@ -223,7 +223,7 @@ struct TilePlan {
 };
 // Tiles along a side of n cells; the first and the last lie against the walls
 // and need no halo there.  0: tiles of this size keep no cell of such a side.
-inline int tile_count(int n, int size, int halo)
+__host__ __device__ inline int tile_count(int n, int size, int halo)
 {
     const int step = size - 2 * halo;
     if (n <= size) return 1;
@@ -244,13 +244,40 @@ struct TileGrid {
 };
 double plan_tiles(const TileGrid *grids, int count, int sms, bool heun, bool per_step,
                   long long steps, TilePlan *best);
+// The tiles of a pass over a batch, in the kernel's parameters: the instances, in
+// the order of their area, lie in n runs, each instance of a run with `tiles`
+// blocks, `across` of them side by side; the run's blocks start at `first`
+// (run[n].first: all blocks), its instances at `place` of the table.
+// Block i << shift belongs to run index[i].  A run is one size (up to 224 of
+// them), or a few sizes of similar area (across 0), whose smaller instances
+// leave some of their blocks idle.  A list in device memory would have to be
+// allocated for every length of a pass, and kept as long as any captured launch
+// that reads it.  20 strips of 400 cells, 1000 steps and 40 reads: 1425 us with a
+// list, 1416 with runs; 256 steps of 129 different grids of up to 311 x 149 take
+// 1223 and 1243 us, of 300 such grids 2626 and 2756.  The parameters stay below
+// 4 KB: beyond that a launch takes the host 5-8 us longer.
+constexpr int kTileRuns = 224, kTileIndex = 64;
+struct TileRun {
+    int first, tiles, place, across;
+};
+struct TileRuns {
+    TileRun run[kTileRuns + 1];
+    int n, shift;
+    unsigned short index[kTileIndex + 1];
+};
+// Whether a side of n cells needs tile i: the tile before it ends short of the
+// wall.
+__host__ __device__ inline bool tile_needed(int i, int n, int size, int halo)
+{
+    return i == 0 || (i - 1) * (size - 2 * halo) + size < n;
+}
 // What a pass runs on: one grid (law, mobility and stage of the arguments not
-// used), or a batch's work list of (instance, tile x, tile y).
+// used), or instances of a batch.
 struct TileLaunch {
     const StepArgs *grid;
-    const void *inst;
-    const int4 *work;
-    int nwork, parity;
+    const void *inst;  // the instance table in the order of the runs
+    const TileRuns *runs;
+    int parity;
     BatchNoise nz;
 };
 cudaError_t launch_tile(int law, int mob, bool per_step, const TileLaunch &a, const TilePlan &p,

@@ -79,25 +79,26 @@ __global__ void __launch_bounds__(32)
 
 template <int LAW, int MOB, bool HEUN>
 __global__ void __launch_bounds__(32)
-    batch_strip_kernel(const InstDev<double> *__restrict__ inst, const int4 *__restrict__ work,
-                       int parity, int stages, int halo)
+    batch_strip_kernel(const InstDev<double> *__restrict__ inst,
+                       const __grid_constant__ TileRuns runs, int parity, int stages, int halo)
 {
-    // the tables are not written while a pass may be queued
-    const int4 w = work[blockIdx.x];
-    const InstDev<double> &I = inst[w.x];
+    // the table is not written while a pass may be queued
+    const batch::TileAt w = batch::tile_of_block(runs, blockIdx.x);
+    const InstDev<double> &I = inst[w.place];
+    if (!tile_needed(w.tile, I.nx, 32, halo)) return;
     const KV<double> k = scalar_kv<double>(make_kv(I.k));
     pass_wait();
     const Ptrs<double> P{I.b[parity], I.n[parity], I.s, nullptr, nullptr, I.b[parity ^ 1],
                          I.n[parity ^ 1]};
-    strip_stages<LAW, MOB, HEUN>(P, I.nx, k, stages, halo, w.y);
+    strip_stages<LAW, MOB, HEUN>(P, I.nx, k, stages, halo, w.tile);
 }
 
 template <int LAW, int MOB, bool HEUN>
 cudaError_t launch_v(const TileLaunch &a, const TilePlan &p, cudaStream_t st)
 {
     if (a.inst)
-        return launch_pass(batch_strip_kernel<LAW, MOB, HEUN>, a.nwork, 32, 0, st,
-                           (const InstDev<double> *)a.inst, a.work, a.parity, p.stages(), p.halo_x());
+        return launch_pass(batch_strip_kernel<LAW, MOB, HEUN>, a.runs->run[a.runs->n].first, 32, 0, st,
+                           (const InstDev<double> *)a.inst, *a.runs, a.parity, p.stages(), p.halo_x());
     const StepArgs &g = *a.grid;
     const Ptrs<double> P{(const double *)g.b, (const double *)g.n, (const double *)g.s, nullptr,
                          nullptr, (double *)g.bo, (double *)g.no};

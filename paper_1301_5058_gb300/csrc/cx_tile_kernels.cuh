@@ -50,22 +50,27 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     one_tile<LAW, MOB, NOISE, HEUN, LX, R>(P, nx, ny, pitch, k, nz, steps, blockIdx.x, blockIdx.y);
 }
 
-// One tile of the batch's work list (instance, tile x, tile y).
+// One tile of an instance of a batch.
 template <int LAW, int MOB, int NOISE, bool HEUN, int LX, int R>
 __global__ void __launch_bounds__(kMaxThreads, 1)
-    batch_tile_kernel(const InstDev<float> *__restrict__ inst, const int4 *__restrict__ work,
-                      int parity, int steps, const long long *step_base, int step_off)
+    batch_tile_kernel(const InstDev<float> *__restrict__ inst,
+                      const __grid_constant__ TileRuns runs, int parity, int steps,
+                      const long long *step_base, int step_off)
 {
-    // the tables are not written while a pass may be queued
-    const int4 w = work[blockIdx.x];
-    const InstDev<float> &I = inst[w.x];
+    // the table is not written while a pass may be queued
+    const batch::TileAt w = batch::tile_of_block(runs, blockIdx.x);
+    const InstDev<float> &I = inst[w.place];
+    const int stages = HEUN ? 2 * steps : steps;
+    const int across = w.across ? w.across : tile_count(I.nx, LX * kCells, x_halo(stages));
+    const int ty = w.tile / across, tx = w.tile - ty * across;
+    if (!tile_needed(ty, I.ny, (int)(blockDim.x / LX) * R, stages)) return;
     const KV<float2> k = make_kv(I.k);
     pass_wait();
     const Ptrs<float> P{I.b[parity], I.n[parity], I.s, nullptr, nullptr, I.b[parity ^ 1],
                         I.n[parity ^ 1]};
     const NoiseT<float> nz =
         NOISE ? inst_noise(I, (uint64_t)(*step_base + step_off)) : NoiseT<float>{};
-    one_tile<LAW, MOB, NOISE, HEUN, LX, R>(P, I.nx, I.ny, I.pitch, k, nz, steps, w.y, w.z);
+    one_tile<LAW, MOB, NOISE, HEUN, LX, R>(P, I.nx, I.ny, I.pitch, k, nz, steps, tx, ty);
 }
 
 template <int LAW, int MOB, int NOISE, bool HEUN, int LX, int R>
@@ -76,8 +81,9 @@ cudaError_t launch_v(const TileLaunch &a, const TilePlan &p, cudaStream_t st)
         auto kern = batch_tile_kernel<LAW, MOB, NOISE, HEUN, LX, R>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        return launch_pass(kern, a.nwork, p.threads, smem, st, (const InstDev<float> *)a.inst, a.work,
-                           a.parity, p.steps, a.nz.step_base, a.nz.step_off);
+        return launch_pass(kern, a.runs->run[a.runs->n].first, p.threads, smem, st,
+                           (const InstDev<float> *)a.inst, *a.runs, a.parity, p.steps, a.nz.step_base,
+                           a.nz.step_off);
     }
     const StepArgs &g = *a.grid;
     const KV<float2> k = make_kv(coef_t<float>(g.k));
