@@ -252,7 +252,8 @@ int cx_set_step(cx_ctx *c, int64_t step);
  * set, cx_step takes several time steps per pass where that is faster and the
  * result the same bits: an FP32 grid of up to about 2500^2 cells (4000^2 with
  * sigma redrawn per step) on tiles that blocks hold in registers, an FP64 strip
- * (ny = 1, static sigma) on one-warp tiles. */
+ * (ny = 1, static sigma) on one-warp tiles.  A height or a depth, the default
+ * ones too, pins the marches until cx_reset_tuning. */
 int cx_set_tile_rows(cx_ctx *c, int32_t rows);
 int cx_get_tile_rows(cx_ctx *c, int32_t *rows);
 
@@ -267,6 +268,15 @@ int cx_get_tile_rows(cx_ctx *c, int32_t *rows);
  * pass is bound by the FP64 pipe).  Errors: INVALID_ARG. */
 int cx_set_time_block(cx_ctx *c, int32_t stages);
 int cx_get_time_block(cx_ctx *c, int32_t *stages);
+
+/* Height and depth as on a new handle: chosen by the library for every call,
+ * several time steps per pass included (cx_set_tile_rows). */
+int cx_reset_tuning(cx_ctx *c);
+
+/* How cx_step(c, n_steps) advances the state, n_steps >= 1: *rows the height of
+ * the marches' tiles, or 0 where the passes run on register tiles or strips;
+ * *steps the most time steps that a pass takes.  Errors: INVALID_ARG. */
+int cx_get_pass(cx_ctx *c, int64_t n_steps, int32_t *rows, int32_t *steps);
 
 /* Write / read a checkpoint: header (grid, params, seed, step, dt,
  * precision) and the raw b, n and sigma arrays.  A run resumed from a

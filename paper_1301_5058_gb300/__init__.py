@@ -102,6 +102,9 @@ _SIGNATURES = {
     "cx_set_tile_rows": (ctypes.c_int, [_P, ctypes.c_int32]),
     "cx_get_tile_rows": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32)]),
     "cx_set_time_block": (ctypes.c_int, [_P, ctypes.c_int32]),
+    "cx_reset_tuning": (ctypes.c_int, [_P]),
+    "cx_get_pass": (ctypes.c_int, [_P, ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
+                                   ctypes.POINTER(ctypes.c_int32)]),
     "cx_batch_set_time_block": (ctypes.c_int, [_P, ctypes.c_int32]),
     "cx_batch_get_time_block": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32)]),
     "cx_get_time_block": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32)]),
@@ -329,6 +332,18 @@ def cx_get_time_block(h) -> int:
     r = ctypes.c_int32()
     _check(lib().cx_get_time_block(h, ctypes.byref(r)))
     return r.value
+
+
+def cx_reset_tuning(h):
+    _check(lib().cx_reset_tuning(h))
+
+
+def cx_get_pass(h, n_steps: int):
+    """(tile rows of the marches, or 0 on register tiles; time steps per pass)
+    of a call of n_steps steps."""
+    r, s = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().cx_get_pass(h, n_steps, ctypes.byref(r), ctypes.byref(s)))
+    return r.value, s.value
 
 
 def cx_batch_set_time_block(h, stages: int):

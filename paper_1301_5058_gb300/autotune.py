@@ -110,32 +110,52 @@ def tune_batch(batch: "cx.Batch", steps: int = 128, reps: int = 3, candidates=No
 
 
 def tune_single(sim: "cx.Sim", steps: int = 20, reps: int = 3, use_cache: bool = True):
-    """Pick the temporal blocking depth and tile height of a single grid's row
-    marches; applies the winner and returns ((time_block, rows), timings).  A
-    grid of up to about 2500^2 cells is faster left alone: without a depth and
-    a height of its own it runs on register tiles (cx_set_tile_rows)."""
+    """Pick the temporal blocking depth and tile height of a single grid, or
+    leave them to the library where that is fastest (register tiles, on grids
+    of up to about 2500^2 cells); applies the winner and returns ((time_block,
+    rows), timings).  The pair that a new handle reports stands for the
+    library's own choice, or for the marches at that depth and height if they
+    were faster.  Only an entry of the cache that compares with the library's
+    choice is used."""
     import torch
     key = f"single/p{sim.params.precision}/s{sim.params.scheme}/n{sim.params.noise_mode}/" \
           f"{sim.grid.nx}x{sim.grid.ny}"
+
+    def apply(choice, automatic):
+        if automatic:
+            cx.cx_reset_tuning(sim.h)
+        else:
+            cx.cx_set_time_block(sim.h, choice[0])
+            cx.cx_set_tile_rows(sim.h, choice[1])
+
     if use_cache:
         hit = _load_cache().get(key)
-        if hit and isinstance(hit.get("choice"), list):
-            cx.cx_set_time_block(sim.h, hit["choice"][0])
-            cx.cx_set_tile_rows(sim.h, hit["choice"][1])
+        if hit and isinstance(hit.get("choice"), list) and "automatic" in hit:
+            apply(hit["choice"], hit["automatic"])
             return tuple(hit["choice"]), {}
     stream = torch.cuda.current_stream()
     cx.cx_set_stream(sim.h, stream.cuda_stream)
-    results = {}
+
+    def measure():
+        sim.step(steps)
+        return _time_steps(torch, stream, sim.step, steps, reps)
+
+    cx.cx_reset_tuning(sim.h)
+    own = (cx.cx_get_time_block(sim.h), cx.cx_get_tile_rows(sim.h))
+    results, automatic = {own: measure()}, True
     for depth in (1, 2):
-        cx.cx_set_time_block(sim.h, depth)
         for rows in SINGLE_CANDIDATES:
             if (sim.grid.ny + rows - 1) // rows > 65535:
                 continue
+            cx.cx_set_time_block(sim.h, depth)
             cx.cx_set_tile_rows(sim.h, rows)
-            sim.step(steps)
-            results[(depth, rows)] = _time_steps(torch, stream, sim.step, steps, reps)
+            t = measure()
+            if (depth, rows) == own:
+                automatic, t = results[own] <= t, min(results[own], t)
+            results[(depth, rows)] = t
     choice = min(results, key=results.get)
-    cx.cx_set_time_block(sim.h, choice[0])
-    cx.cx_set_tile_rows(sim.h, choice[1])
-    _store(key, {"choice": list(choice), "us_per_step": results[choice] * 1e6})
+    automatic = automatic and choice == own
+    apply(choice, automatic)
+    _store(key, {"choice": list(choice), "automatic": automatic,
+                 "us_per_step": results[choice] * 1e6})
     return choice, results

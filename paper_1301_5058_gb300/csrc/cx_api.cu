@@ -144,6 +144,11 @@ struct FieldBuffers {
     long long pitch;  // elements per row
 };
 
+// Two stages per pass pay off for an FP32 state, whose pass is bound by memory
+// and instruction issue; the FP64 pass is bound by the FP64 pipe and the fused
+// pass's overlap lanes only add FP64 work.
+int default_time_block(int prec) { return prec == CX_PREC_F32 ? 2 : 1; }
+
 // Allocate the handle and its buffers, or adopt the caller's field arrays
 // (contents: zero).
 int alloc_ctx(const cx_grid *g, const cx_params *p, uint64_t seed, double dt, cx_ctx **out,
@@ -162,10 +167,7 @@ int alloc_ctx(const cx_grid *g, const cx_params *p, uint64_t seed, double dt, cx
     c->own_fields = ext ? 0 : 1;
     c->dt = dt;
     c->tile_rows = 0;  // automatic (auto_tile_rows)
-    // two stages per pass pay off for an FP32 state, whose pass is bound by
-    // memory and instruction issue; the FP64 pass is bound by the FP64 pipe
-    // and the fused pass's overlap lanes only add FP64 work
-    c->time_block = c->prec == CX_PREC_F32 ? 2 : 1;
+    c->time_block = default_time_block(c->prec);
     c->stream = nullptr;
     cudaGetDevice(&c->device);
     c->num_sms = 0;
@@ -886,6 +888,29 @@ int cx_set_time_block(cx_ctx *c, int32_t stages)
         return fail(CX_ERR_INVALID_ARG, "time block %d: must be 1 or 2 stages per pass", stages);
     c->time_block = stages;
     c->depth_set = 1;
+    return CX_OK;
+}
+
+int cx_reset_tuning(cx_ctx *c)
+{
+    int rc = check_ctx(c);
+    if (rc) return rc;
+    c->tile_rows = 0;
+    c->time_block = default_time_block(c->prec);
+    c->depth_set = 0;
+    return CX_OK;
+}
+
+int cx_get_pass(cx_ctx *c, int64_t n_steps, int32_t *rows, int32_t *steps)
+{
+    int rc = check_ctx(c);
+    if (rc) return rc;
+    if (!rows || !steps || n_steps < 1)
+        return fail(CX_ERR_INVALID_ARG, "need rows, steps and n_steps >= 1");
+    const bool tiles = use_tiles(c, n_steps);
+    const bool two = c->time_block == 2 && c->p.scheme == CX_SCHEME_EULER && n_steps >= 2;
+    *rows = tiles ? 0 : tile_rows_of(c);
+    *steps = tiles ? c->plan.steps : two ? 2 : 1;
     return CX_OK;
 }
 
