@@ -314,12 +314,13 @@ int cx_batch_set_stream(cx_batch *b, void *stream);
 
 /* Performance knobs, none of which changes any result bit:
  *   tile_rows   rows per tile of the step kernel (1..4096; the tiles of
- *               both depths; default 128 for FP32 batches, which take two
- *               stages per pass, 32 for FP64 ones).  With the height,
- *               the groups, the resident mode and the depth all at their
- *               defaults the batch chooses for itself, as a single grid does:
- *               fewer rows where it would leave the GPU idle, or several
- *               steps per pass on register tiles;
+ *               both depths).  A new batch reports 128 (FP32, which takes two
+ *               stages per pass) or 32 (FP64) and chooses for itself, as a
+ *               single grid does: fewer rows where that keeps the GPU busier,
+ *               or several steps per pass on register tiles
+ *               (cx_batch_get_pass).  From this call or
+ *               cx_batch_set_time_block on, the default values included, the
+ *               marches run as told, until cx_batch_reset_tuning;
  *   graph_steps steps captured per CUDA graph and replayed (0: plain
  *               launches; rounded up to even for Euler; default 64);
  *   group_bytes if > 0, instances are cut into consecutive groups whose
@@ -347,6 +348,16 @@ int cx_batch_get_tuning(cx_batch *b, int32_t *tile_rows, int32_t *graph_steps, i
  * Errors: INVALID_ARG. */
 int cx_batch_set_time_block(cx_batch *b, int32_t stages);
 int cx_batch_get_time_block(cx_batch *b, int32_t *stages);
+
+/* All knobs as on a new batch, but for graph_steps (as in cx_batch_set_tuning,
+ * 64 on a new batch): the batch chooses for itself again.  Errors: INVALID_ARG,
+ * CUDA, OOM. */
+int cx_batch_reset_tuning(cx_batch *b, int32_t graph_steps);
+
+/* How cx_batch_step(b, n_steps) advances the batch, as cx_get_pass: *rows the
+ * height in effect of the marches' tiles, or 0 where the passes run on register
+ * tiles or strips; *steps the most time steps that a pass takes. */
+int cx_batch_get_pass(cx_batch *b, int64_t n_steps, int32_t *rows, int32_t *steps);
 
 /* Advance every instance by n_steps >= 0 steps.  Asynchronous.  A call of fewer
  * than graph_steps steps (any call if graph_steps is 0) is launches alone, of

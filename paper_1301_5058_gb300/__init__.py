@@ -105,6 +105,9 @@ _SIGNATURES = {
     "cx_reset_tuning": (ctypes.c_int, [_P]),
     "cx_get_pass": (ctypes.c_int, [_P, ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
                                    ctypes.POINTER(ctypes.c_int32)]),
+    "cx_batch_reset_tuning": (ctypes.c_int, [_P, ctypes.c_int32]),
+    "cx_batch_get_pass": (ctypes.c_int, [_P, ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
+                                         ctypes.POINTER(ctypes.c_int32)]),
     "cx_batch_set_time_block": (ctypes.c_int, [_P, ctypes.c_int32]),
     "cx_batch_get_time_block": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32)]),
     "cx_get_time_block": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32)]),
@@ -377,6 +380,17 @@ def cx_batch_set_tuning(h, tile_rows: int, graph_steps: int, group_bytes: int,
     _check(lib().cx_batch_set_tuning(h, tile_rows, graph_steps, group_bytes, resident_steps))
 
 
+def cx_batch_reset_tuning(h, graph_steps: int = 64):
+    _check(lib().cx_batch_reset_tuning(h, graph_steps))
+
+
+def cx_batch_get_pass(h, n_steps: int):
+    """As cx_get_pass, of a batch's call of n_steps steps."""
+    r, s = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().cx_batch_get_pass(h, n_steps, ctypes.byref(r), ctypes.byref(s)))
+    return r.value, s.value
+
+
 def cx_batch_get_tuning(h):
     r, g, b, s = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int64(), ctypes.c_int32()
     _check(lib().cx_batch_get_tuning(h, ctypes.byref(r), ctypes.byref(g), ctypes.byref(b),
@@ -643,6 +657,11 @@ class Batch:
         cx_batch_set_field(self.h, index, which, arr)
 
     def tune(self, tile_rows, graph_steps, group_bytes, resident_steps=0, time_block=None):
+        """Pin the knobs (cx_batch_set_tuning, cx_batch_set_time_block), or give
+        all but graph_steps back to the library: tune(0, graph_steps, 0, 0, 0)."""
+        if (tile_rows, group_bytes, resident_steps, time_block) == (0, 0, 0, 0):
+            cx_batch_reset_tuning(self.h, graph_steps)
+            return
         cx_batch_set_tuning(self.h, tile_rows, graph_steps, group_bytes, resident_steps)
         if time_block is not None:
             cx_batch_set_time_block(self.h, time_block)

@@ -21,11 +21,13 @@ import paper_1301_5058_gb300 as cx
 L2_BYTES = 126 * 2 ** 20   # GB300 L2 (about 126 MiB usable)
 
 # (tile rows, graph steps, group bytes, resident steps, stages per pass):
-# one launch per pass over every instance at either depth; L2-sized groups
-# stepped by resident launches (one stage per pass) are searched only when
-# asked for (RESIDENT_CANDIDATES: they have never won on GB300)
-BATCH_CANDIDATES = [(rows, graph, 0, 0, depth) for depth in (1, 2) for rows in (16, 32, 64, 128)
-                    for graph in (0, 64)]
+# what the library chooses for itself, then one launch per pass over every
+# instance at either depth; L2-sized groups stepped by resident launches (one
+# stage per pass) are searched only when asked for (RESIDENT_CANDIDATES: they
+# have never won on GB300)
+AUTOMATIC = (0, 64, 0, 0, 0)
+BATCH_CANDIDATES = [AUTOMATIC] + [(rows, graph, 0, 0, depth) for depth in (1, 2)
+                                  for rows in (16, 32, 64, 128) for graph in (0, 64)]
 RESIDENT_CANDIDATES = [(rows, 0, group, res, 1) for rows in (4, 8, 16)
                        for group in (L2_BYTES // 2, L2_BYTES // 4) for res in (50, 200)]
 SINGLE_CANDIDATES = (2, 4, 8, 16, 32, 64, 128, 256)
@@ -78,13 +80,15 @@ def _time_steps(torch, stream, fn, steps: int, reps: int) -> float:
 def tune_batch(batch: "cx.Batch", steps: int = 128, reps: int = 3, candidates=None,
                use_cache: bool = True, verbose: bool = False):
     """Pick (tile_rows, graph_steps, group_bytes, resident_steps, stages per
-    pass) for `batch`, apply it and return (choice, {candidate: seconds per
-    step}).  The timed steps advance the batch's state."""
+    pass) for `batch`, or AUTOMATIC (its rows and stages 0) where the library's
+    own choice is fastest; apply it and return (choice, {candidate: seconds per
+    step}).  The timed steps advance the batch's state.  Without candidates of
+    one's own, only an entry of the cache that compares with AUTOMATIC is used."""
     import torch
     key = batch_key(batch.grids, batch.params)
     if use_cache:
         hit = _load_cache().get(key)
-        if hit:
+        if hit and (candidates or hit.get("automatic")):
             choice = tuple(hit["choice"])
             batch.tune(*choice)
             return choice, {}
@@ -105,7 +109,8 @@ def tune_batch(batch: "cx.Batch", steps: int = 128, reps: int = 3, candidates=No
                   f"resident={cand[3]:4d} depth={cand[4]}: {results[cand] * 1e6:9.1f} us/step")
     choice = min(results, key=results.get)
     batch.tune(*choice)
-    _store(key, {"choice": list(choice), "us_per_step": results[choice] * 1e6})
+    _store(key, {"choice": list(choice), "automatic": AUTOMATIC in results,
+                 "us_per_step": results[choice] * 1e6})
     return choice, results
 
 

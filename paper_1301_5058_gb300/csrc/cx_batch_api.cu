@@ -60,7 +60,7 @@ struct cx_batch {
     std::vector<int> work2_begin;
     int rows = 32;                  // tile height set, or reported as the default
     int march_rows = 32;            // tile height in effect
-    bool tuned = false;             // a knob of the marches is off its default: they run as told
+    bool tuned = false;             // a knob of the marches was set: they run as told
     int num_sms = 1;
     std::vector<cx::TileGrid> sizes;  // the instances' distinct sizes
     int64_t plan_for = 0;           // steps that `plan` was made for (0: none yet)
@@ -187,21 +187,22 @@ int auto_rows(const cx_batch *B)
 
 void build_groups(cx_batch *B);
 
-// Whether the knobs choose a march: the height, the depth, the groups or the
-// resident mode differ from the defaults.
-bool is_tuned(const cx_batch *B)
+int default_rows(int prec) { return prec == CX_PREC_F32 ? 128 : 32; }
+int default_time_block(int prec) { return prec == CX_PREC_F32 ? 2 : 1; }  // as a single grid
+
+int even_for_euler(const cx_batch *B, int graph_steps)
 {
-    const bool f32 = B->prec == CX_PREC_F32;
-    return B->rows != (f32 ? 128 : 32) || B->time_block != (f32 ? 2 : 1) || B->group_bytes > 0 ||
-           B->resident_steps > 0;
+    return B->scheme == CX_SCHEME_EULER && (graph_steps & 1) ? graph_steps + 1 : graph_steps;
 }
 
-// After a knob was set: the height in effect, and the marches' work lists.
-int apply_tuning(cx_batch *B)
+// After a knob was set (`tuned`) or all were given back: the height in effect,
+// and the marches' work lists.
+int apply_tuning(cx_batch *B, bool tuned)
 {
-    B->tuned = is_tuned(B);
+    B->tuned = tuned;
     B->plan_for = 0;
-    const int rows = B->tuned ? B->rows : auto_rows(B);
+    B->tiles = false;
+    const int rows = tuned ? B->rows : auto_rows(B);
     if (rows != B->march_rows) {
         B->march_rows = rows;
         const int rc = build_work(B);
@@ -237,6 +238,13 @@ bool use_tiles(cx_batch *B, int64_t steps)
         B->plan_for = steps;
     }
     return B->tiles;
+}
+
+// The steps that a call of n_steps plans for: a graph's if it replays one (and
+// the rest by the same plan).
+int64_t run_length(const cx_batch *B, int64_t n_steps)
+{
+    return B->graph_steps > 0 && n_steps >= B->graph_steps ? B->graph_steps : n_steps;
 }
 
 // Steps of the next register-tile pass of `left`: as few passes as the plan
@@ -464,11 +472,11 @@ int cx_batch_create(int32_t count, const cx_grid *grids, const cx_params *params
     B->mob = params[0].mobility;
     B->scheme = params[0].scheme;
     B->noise = params[0].noise_mode == CX_NOISE_PER_STEP ? 1 : 0;
-    B->time_block = B->prec == CX_PREC_F32 ? 2 : 1;  // as a single grid
+    B->time_block = default_time_block(B->prec);
     // Two stages per pass recompute 4 halo rows per tile: 128-row tiles keep
     // that to 3 % (1024 instances of 1024^2: 5.6e11 cell-updates/s against
     // 4.6e11 with 32-row tiles; 64 to 256 rows within 2 % of the best)
-    B->rows = B->time_block == 2 ? 128 : 32;
+    B->rows = default_rows(B->prec);
     B->elem = B->prec == CX_PREC_F64 ? sizeof(double) : sizeof(float);
     B->g.assign(grids, grids + count);
     B->p.assign(params, params + count);
@@ -595,10 +603,39 @@ int cx_batch_set_tuning(cx_batch *B, int32_t tile_rows, int32_t graph_steps, int
     BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before retuning");
     drop_graphs(B);
     B->rows = tile_rows;
-    B->graph_steps = (B->scheme == CX_SCHEME_EULER && (graph_steps & 1)) ? graph_steps + 1 : graph_steps;
+    B->graph_steps = even_for_euler(B, graph_steps);
     B->group_bytes = group_bytes;
     B->resident_steps = resident_steps;
-    return apply_tuning(B);
+    return apply_tuning(B, true);
+}
+
+int cx_batch_reset_tuning(cx_batch *B, int32_t graph_steps)
+{
+    int rc = check_batch(B);
+    if (rc) return rc;
+    if (graph_steps < 0 || graph_steps > 100000) return bfail(CX_ERR_INVALID_ARG, "graph_steps 0..100000");
+    BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before retuning");
+    drop_graphs(B);
+    B->rows = default_rows(B->prec);
+    B->time_block = default_time_block(B->prec);
+    B->graph_steps = even_for_euler(B, graph_steps);
+    B->group_bytes = 0;
+    B->resident_steps = 0;
+    return apply_tuning(B, false);
+}
+
+int cx_batch_get_pass(cx_batch *B, int64_t n_steps, int32_t *rows, int32_t *steps)
+{
+    int rc = check_batch(B);
+    if (rc) return rc;
+    if (!rows || !steps || n_steps < 1)
+        return bfail(CX_ERR_INVALID_ARG, "need rows, steps and n_steps >= 1");
+    const bool tiles = use_tiles(B, run_length(B, n_steps));
+    const bool two = B->time_block == 2 && B->scheme == CX_SCHEME_EULER && B->resident_steps == 0 &&
+                     n_steps >= 2;
+    *rows = tiles ? 0 : B->march_rows;
+    *steps = tiles ? B->plan.steps : two ? 2 : 1;
+    return CX_OK;
 }
 
 int cx_batch_get_tuning(cx_batch *B, int32_t *tile_rows, int32_t *graph_steps, int64_t *group_bytes,
@@ -622,7 +659,7 @@ int cx_batch_set_time_block(cx_batch *B, int32_t stages)
     BX_CUDA(cudaStreamSynchronize(B->stream), "synchronize before retuning");
     drop_graphs(B);
     B->time_block = stages;
-    return apply_tuning(B);
+    return apply_tuning(B, true);
 }
 
 int cx_batch_get_time_block(cx_batch *B, int32_t *stages)
@@ -641,9 +678,8 @@ int cx_batch_step(cx_batch *B, int64_t n_steps)
     if (rc) return rc;
     if (n_steps < 0) return bfail(CX_ERR_INVALID_ARG, "n_steps < 0");
     if (n_steps == 0) return CX_OK;
-    const bool whole = B->graph_steps > 0 && n_steps >= B->graph_steps;  // at least one graph
     // (the graphs hold the plan for graph_steps, which only a knob changes)
-    B->tiles = use_tiles(B, whole ? B->graph_steps : n_steps);
+    B->tiles = use_tiles(B, run_length(B, n_steps));
     const int ngroups = (int)B->group_first.size() - 1;
     if (B->graph_steps > 0 && (int)B->gexec[0].size() != ngroups) {
         drop_graphs(B);

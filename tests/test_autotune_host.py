@@ -81,3 +81,34 @@ def test_single_entries_without_the_librarys_choice_are_not_used(tuner):
     lib = tuner(FakeLib({None: 0.5}, (2, 4)))
     assert autotune.tune_single(sim_of(1024), use_cache=True)[0] == (2, 4)
     assert lib.force is None
+
+
+class FakeBatch:
+    def __init__(self, timings):
+        self.timings, self.force, self._stream, self.h = timings, None, object(), 1
+        self.grids = [types.SimpleNamespace(nx=256, ny=256)] * 3
+        self.params = [types.SimpleNamespace(precision=1, scheme=0)] * 3
+
+    def tune(self, *knobs):
+        self.force = knobs
+
+    def step(self, n):
+        pass
+
+
+@pytest.mark.parametrize("timings,choice", [
+    ({autotune.AUTOMATIC: 0.5}, autotune.AUTOMATIC),
+    ({autotune.AUTOMATIC: 0.5, (128, 64, 0, 0, 2): 0.4}, (128, 64, 0, 0, 2))])
+def test_batch_candidates_include_the_librarys_choice(tuner, monkeypatch, timings, choice):
+    bt = FakeBatch(timings)
+    monkeypatch.setattr(autotune, "_time_steps", lambda *a: bt.timings.get(bt.force, 1.0))
+    got, results = autotune.tune_batch(bt)
+    assert got == choice == bt.force and set(results) == set(autotune.BATCH_CANDIDATES)
+    bt.force = None
+    assert autotune.tune_batch(bt) == (choice, {}) and bt.force == choice
+    # an entry that never compared with the library's choice is not used
+    tuner.cache.write_text(json.dumps({autotune.batch_key(bt.grids, bt.params):
+                                       {"choice": [16, 0, 0, 0, 1]}}))
+    assert autotune.tune_batch(bt)[0] == choice
+    # of a caller's own candidates the fastest, the library's choice or not
+    assert autotune.tune_batch(bt, candidates=[(16, 0, 0, 0, 1)], use_cache=False)[0] == (16, 0, 0, 0, 1)

@@ -45,3 +45,43 @@ def test_a_tuned_small_grid_still_runs_on_tiles(cx, tmp_path, monkeypatch):
         for _ in range(2):  # timed, then from the cache
             autotune.tune_single(sim, steps=32, reps=3)
             assert cx.cx_get_pass(sim.h, 64)[0] == 0
+
+
+@pytest.mark.parametrize("size,prec,rows,depth", [((256, 256), 1, 128, 2), ((400, 1), 0, 32, 1)])
+def test_batch_knobs_pin_the_marches_at_their_defaults_too(cx, size, prec, rows, depth):
+    kw = dict(BASE, precision=prec, chemo_law=1 - prec)
+    dtype = np.float32 if prec else np.float64
+    specs = [dict(nx=size[0], ny=size[1], dx=1.0, seed=i, **kw) for i in range(4)]
+    with cx.Batch(specs) as bt, cx.Batch(specs) as ref:
+        assert cx.cx_batch_get_pass(bt.h, 64)[0] == 0 and cx.cx_batch_get_pass(bt.h, 64)[1] > 2
+        for pin in (lambda: bt.tune(rows, 64, 0, 0, depth), lambda: bt.tune(rows, 32, 0),
+                    lambda: cx.cx_batch_set_time_block(bt.h, depth)):
+            pin()
+            assert cx.cx_batch_get_tuning(bt.h)[0] == rows
+            assert cx.cx_batch_get_pass(bt.h, 64) == (rows, depth)
+            bt.step(70)
+            bt.tune(0, 64, 0, 0, 0)
+            assert cx.cx_batch_get_tuning(bt.h) == (rows, 64, 0, 0)
+            assert cx.cx_batch_get_time_block(bt.h) == depth
+            assert cx.cx_batch_get_pass(bt.h, 64)[0] == 0
+            bt.step(70)
+        bt.tune(7, 0, 0, 5)  # the resident mode: one stage per pass
+        assert cx.cx_batch_get_pass(bt.h, 64) == (7, 1)
+        bt.step(9)
+        ref.step(6 * 70 + 9)
+        for i in range(4):
+            assert np.array_equal(bt.field(i, cx.CX_FIELD_B, dtype), ref.field(i, cx.CX_FIELD_B, dtype))
+        for bad in (-1, 100001):
+            with pytest.raises(cx.CxError):
+                cx.cx_batch_reset_tuning(bt.h, bad)
+
+
+def test_height_in_effect_of_an_untouched_batch(cx):
+    # the sweep's mix of sizes stays on the marches: 64 rows, whatever the
+    # reported default
+    from paper_1301_5058_gb300 import workloads as W
+    with cx.Batch(W.sweep_specs(24, seed=0, steps=100)) as bt:
+        assert cx.cx_batch_get_tuning(bt.h)[0] == 128
+        assert cx.cx_batch_get_pass(bt.h, 64) == (64, 2)
+        bt.tune(128, 64, 0, 0, 2)
+        assert cx.cx_batch_get_pass(bt.h, 64) == (128, 2)
