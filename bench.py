@@ -600,7 +600,9 @@ def oracle_error_grid(spec, nx=288, ny=200, steps=ORACLE_CHECK_STEPS):
 
 def oracle_error_sweep(tuning, steps=ORACLE_CHECK_STEPS):
     """The batch path with the sweep's tuning, on three instances of the
-    sweep's kind (smaller sides, one ragged), each against the oracle."""
+    sweep's kind (smaller sides, one ragged), each against the oracle.  The
+    tuning pins the march that the sweep runs on, which instances this small
+    would leave for register tiles."""
     import paper_1301_5058_gb300 as cx
     from paper_1301_5058_gb300 import workloads as W
     specs = W.sweep_specs(3, seed=0, steps=steps)
@@ -611,6 +613,8 @@ def oracle_error_sweep(tuning, steps=ORACLE_CHECK_STEPS):
     with cx.Batch(specs) as bt:
         bt.tune(tuning["tile_rows"], tuning["graph_steps"], tuning["group_bytes"],
                 tuning["resident_steps"], tuning["time_block"])
+        march = cx.cx_batch_get_pass(bt.h, steps)
+        assert march == (tuning["tile_rows"], tuning["time_block"]), march
         refs = []
         for i, sp in enumerate(specs):
             cfg = dict(W.CONFIG1, **{k: v for k, v in sp.items() if k != "precision"})
@@ -625,7 +629,8 @@ def oracle_error_sweep(tuning, steps=ORACLE_CHECK_STEPS):
     return {"rel_l2_b": worst[0], "rel_l2_n": worst[1], "tolerance": 1e-4,
             "pass": max(worst) <= 1e-4,
             "case": f"3 instances (160^2, 224^2, 97^2) of the sweep's kind, {steps} steps, "
-                    "the sweep's tuning, worst instance"}
+                    f"the sweep's march ({march[0]}-row tiles, {march[1]} stages per pass), "
+                    "worst instance"}
 
 
 def measure_alu_peaks():
@@ -836,12 +841,14 @@ def sweep_record(args):
     create_s = time.perf_counter() - t0
     cx.cx_batch_set_stream(bt.h, stream.cuda_stream)
     bt._stream = stream
+    # the record describes the marches, so they are pinned at every --count
     if args.tune:
-        autotune.tune_batch(bt, steps=64, reps=2, use_cache=False)
+        autotune.tune_batch(bt, steps=64, reps=2, use_cache=False,
+                            candidates=[c for c in autotune.BATCH_CANDIDATES if c != autotune.AUTOMATIC])
     else:
-        # the autotuner's choice on this sweep (128-row tiles, 64-step graphs,
-        # two stages per pass), fixed so that the default run needs no search
-        bt.tune(128, 64, 0, 0, 2)
+        # what an untouched batch of this sweep runs on: 64-row tiles, 64-step
+        # graphs, two stages per pass
+        bt.tune(64, 64, 0, 0, 2)
     choice = cx.cx_batch_get_tuning(bt.h)
     depth = cx.cx_batch_get_time_block(bt.h)
 
