@@ -415,7 +415,7 @@ int check_barrier(cx_batch *B)
     BX_CUDA(cudaMemcpy(&err, (char *)B->d_barrier + 8, sizeof err, cudaMemcpyDeviceToHost),
             "barrier flag read");
     if (err) {
-        BX_CUDA(cudaMemset((char *)B->d_barrier + 8, 0, sizeof err), "barrier flag reset");
+        BX_CUDA(cudaMemsetAsync((char *)B->d_barrier + 8, 0, sizeof err, B->stream), "barrier flag reset");
         return bfail(CX_ERR_TIMEOUT, "a grid barrier wait of the resident batch kernel ran out; "
                                      "the batch state is undefined");
     }

@@ -986,7 +986,8 @@ int cx_mlp_create_members(int32_t max_batch, int32_t members, cx_mlp **out)
     cudaError_t e = cudaStreamCreateWithFlags(&m->st, cudaStreamNonBlocking);
     auto A = [&](void **p, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(p, bytes);
-        if (e == cudaSuccess) e = cudaMemset(*p, 0, bytes);
+        // on the network's own stream: nothing orders its work after the legacy one's
+        if (e == cudaSuccess) e = cudaMemsetAsync(*p, 0, bytes, m->st);
     };
     A((void **)&m->P, E * NPARAM * 4); A((void **)&m->G, E * NPARAM * 4);
     A((void **)&m->M, E * NPARAM * 4); A((void **)&m->V, E * NPARAM * 4);
