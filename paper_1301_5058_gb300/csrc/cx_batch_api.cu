@@ -121,30 +121,42 @@ cudaError_t upload(cx_batch *B, void *dst, const void *src, size_t bytes)
     return e == cudaSuccess ? cudaStreamSynchronize(B->stream) : e;
 }
 
-// Tile work lists for the current tile height, instance by instance: the
-// one-stage march's tiles and the two-stage march's 120-column
-// tiles.
-int build_work(cx_batch *B)
+// Tile work lists for tiles of `rows` rows, instance by instance: the one-stage
+// march's tiles and the two-stage march's 120-column tiles.  If one cannot be
+// made, the height and the lists in effect stay.
+int build_work(cx_batch *B, int rows)
 {
-    for (int f = 0; f < 2; ++f) {
+    int4 *d[2] = {nullptr, nullptr};
+    std::vector<int> begin[2];
+    cudaError_t e = cudaSuccess;
+    for (int f = 0; f < 2 && e == cudaSuccess; ++f) {
         const int cols = f ? kFusedTileCols : tile_cols(B->prec);
-        std::vector<int> &begin = f ? B->work2_begin : B->work_begin;
-        int4 *&d = f ? B->d_work2 : B->d_work;
         std::vector<int4> w;
-        begin.assign(B->count + 1, 0);
+        begin[f].assign(B->count + 1, 0);
         for (int i = 0; i < B->count; ++i) {
-            begin[i] = (int)w.size();
+            begin[f][i] = (int)w.size();
             const int tx = (B->g[i].nx + cols - 1) / cols;
-            const int ty = (B->g[i].ny + B->march_rows - 1) / B->march_rows;
+            const int ty = (B->g[i].ny + rows - 1) / rows;
             for (int y = 0; y < ty; ++y)
                 for (int x = 0; x < tx; ++x) w.push_back(make_int4(i, x, y, 0));
         }
-        begin[B->count] = (int)w.size();
-        if (d) cudaFree(d);
-        d = nullptr;
-        BX_CUDA(cudaMalloc((void **)&d, w.size() * sizeof(int4)), "work list allocation");
-        BX_CUDA(upload(B, d, w.data(), w.size() * sizeof(int4)), "work list upload");
+        begin[f][B->count] = (int)w.size();
+        e = cudaMalloc((void **)&d[f], w.size() * sizeof(int4));
+        if (e == cudaSuccess) e = upload(B, d[f], w.data(), w.size() * sizeof(int4));
     }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        for (int4 *p : d)
+            if (p) cudaFree(p);
+        return bcuda(e, "tile work lists");
+    }
+    if (B->d_work) cudaFree(B->d_work);
+    if (B->d_work2) cudaFree(B->d_work2);
+    B->d_work = d[0];
+    B->d_work2 = d[1];
+    B->work_begin.swap(begin[0]);
+    B->work2_begin.swap(begin[1]);
+    B->march_rows = rows;
     return CX_OK;
 }
 
@@ -202,14 +214,9 @@ int apply_tuning(cx_batch *B, bool tuned)
     B->tuned = tuned;
     B->plan_for = 0;
     B->tiles = false;
-    const int rows = tuned ? B->rows : auto_rows(B);
-    if (rows != B->march_rows) {
-        B->march_rows = rows;
-        const int rc = build_work(B);
-        if (rc) return rc;
-    }
     build_groups(B);
-    return CX_OK;
+    const int rows = tuned ? B->rows : auto_rows(B);
+    return rows == B->march_rows ? CX_OK : build_work(B, rows);
 }
 
 // Whether runs of `steps` steps take several steps per pass, as a single grid
@@ -558,8 +565,7 @@ int cx_batch_create(int32_t count, const cx_grid *grids, const cx_params *params
         cudaGetLastError();
         B->num_sms = 1;  // only the choice of tiles uses it
     }
-    B->march_rows = auto_rows(B);
-    int rc = build_work(B);
+    int rc = build_work(B, auto_rows(B));
     if (rc) { free_batch(B); return rc; }
     build_groups(B);
     // initial state of every instance
