@@ -252,17 +252,18 @@ double plan_tiles(const TileGrid *grids, int count, int sms, bool heun, bool per
 // them), or a few sizes of similar area (across 0), whose smaller instances
 // leave some of their blocks idle.  A list in device memory would have to be
 // allocated for every length of a pass, and kept as long as any captured launch
-// that reads it.  20 strips of 400 cells, 1000 steps and 40 reads: 1425 us with a
-// list, 1416 with runs; 256 steps of 129 different grids of up to 311 x 149 take
-// 1223 and 1243 us, of 300 such grids 2626 and 2756.  The parameters stay below
-// 4 KB: beyond that a launch takes the host 5-8 us longer.
+// that reads it.  Lists and runs: 20 strips of 400 cells, 1000 steps and 40
+// reads, 1431 and 1422 us; per step 96 instances of 256^2 13.46 and 13.50, 40 of
+// 300^2 with Heun 21.09 and 21.32; 256 steps of 129 different grids of up to
+// 311 x 149 1225 and 1240, of 300 such grids 2630 and 2733.  The parameters stay
+// below 4 KB: beyond that a launch takes the host 5-8 us longer.
 constexpr int kTileRuns = 224, kTileIndex = 64;
 struct TileRun {
     int first, tiles, place, across;
 };
 struct TileRuns {
-    TileRun run[kTileRuns + 1];
     int n, shift;
+    TileRun run[kTileRuns + 1];
     unsigned short index[kTileIndex + 1];
 };
 // Whether a side of n cells needs tile i: the tile before it ends short of the

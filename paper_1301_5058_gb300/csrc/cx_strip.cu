@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(32)
     // the table is not written while a pass may be queued
     const batch::TileAt w = batch::tile_of_block(runs, blockIdx.x);
     const InstDev<double> &I = inst[w.place];
-    if (!tile_needed(w.tile, I.nx, 32, halo)) return;
+    if (!w.across && !tile_needed(w.tile, I.nx, 32, halo)) return;
     const KV<double> k = scalar_kv<double>(make_kv(I.k));
     pass_wait();
     const Ptrs<double> P{I.b[parity], I.n[parity], I.s, nullptr, nullptr, I.b[parity ^ 1],

@@ -62,8 +62,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     const InstDev<float> &I = inst[w.place];
     const int stages = HEUN ? 2 * steps : steps;
     const int across = w.across ? w.across : tile_count(I.nx, LX * kCells, x_halo(stages));
-    const int ty = w.tile / across, tx = w.tile - ty * across;
-    if (!tile_needed(ty, I.ny, (int)(blockDim.x / LX) * R, stages)) return;
+    const int ty = batch::quotient(w.tile, across), tx = w.tile - ty * across;
+    if (!w.across && !tile_needed(ty, I.ny, (int)(blockDim.x / LX) * R, stages)) return;
     const KV<float2> k = make_kv(I.k);
     pass_wait();
     const Ptrs<float> P{I.b[parity], I.n[parity], I.s, nullptr, nullptr, I.b[parity ^ 1],
