@@ -16,7 +16,8 @@
 //   forward_kernel   H1 is computed while the A operand is staged, the
 //                    256-wide product runs on tcgen05 with its accumulator
 //                    in tensor memory, and in the epilogue each thread owns
-//                    one batch row: H2, Y, dY, the row's loss and dZ2;
+//                    16 columns of one batch row: H2, dZ2 and, in the first
+//                    thread of a row, Y, dY and the row's loss;
 //   backward_kernel  the dH1 tiles (epilogue: dZ1) and the dW2 tiles, on
 //                    tcgen05;
 //   column_sums      the thin-layer and bias gradients and the loss, in a
@@ -562,9 +563,9 @@ __global__ void __launch_bounds__(kThreads, 2) __cluster_dims__(kSplit, 1, 1)
 // Forward pass alone on many rows: batch rows [128 i, 128 i + 128) of member
 // blockIdx.y, i = blockIdx.x, all 256 columns in one CTA, whose H1 needs no
 // other CTA.  With more tiles than the GPU holds at a time throughput counts,
-// not a tile's latency: a call of 8 members x 8192 rows takes 99 us (clusters
-// 125; with the whole shared memory per CTA, one per SM, 104), while at 8 x 1024
-// rows the clusters take 41 (51).  Same sums in the same order as the clusters
+// not a tile's latency: a call of 8 members x 8192 rows takes 91 us (clusters
+// 115; 4096 rows 57 and 70; 2048 rows 43 and 46), while at 8 x 1024 rows the
+// clusters take 32 (whole tiles 43).  Same sums in the same order as the clusters
 // (a thread sums one quarter of a row).
 constexpr int kWideKC = 128;
 constexpr int kWideA = kRows * kWideKC * 2, kWideB = H * kWideKC * 2;
