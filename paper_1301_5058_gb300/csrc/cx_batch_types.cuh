@@ -57,16 +57,16 @@ struct TileAt {
 };
 __device__ __forceinline__ TileAt tile_of_block(const TileRuns &z, int blk)
 {
-    int k = 0;
-    if (z.n > 1) {  // (one size: 96 instances of 256^2 13.53 -> 13.50 us per step)
-        const int i0 = blk >> z.shift;
-        int last = z.index[i0 + 1];
-        k = z.index[i0];
-        while (k < last) {
-            const int mid = (k + last + 1) / 2;
-            if (blk < z.run[mid].first) last = mid - 1;
-            else k = mid;
-        }
+    int k = 0, last = z.n - 1;
+    if (z.n > 8) {  // (fewer lie together, in the first lines of the parameters)
+        const int i = blk >> z.shift;
+        k = z.index[i];
+        last = z.index[i + 1];
+    }
+    while (k < last) {
+        const int mid = (k + last + 1) / 2;
+        if (blk < z.run[mid].first) last = mid - 1;
+        else k = mid;
     }
     const TileRun r = z.run[k];
     const int t = blk - r.first, i = quotient(t, r.tiles);

@@ -253,10 +253,11 @@ double plan_tiles(const TileGrid *grids, int count, int sms, bool heun, bool per
 // leave some of their blocks idle.  A list in device memory would have to be
 // allocated for every length of a pass, and kept as long as any captured launch
 // that reads it.  Lists and runs: 20 strips of 400 cells, 1000 steps and 40
-// reads, 1431 and 1422 us; per step 96 instances of 256^2 13.46 and 13.50, 40 of
-// 300^2 with Heun 21.09 and 21.32; 256 steps of 129 different grids of up to
-// 311 x 149 1225 and 1240, of 300 such grids 2630 and 2733.  The parameters stay
-// below 4 KB: beyond that a launch takes the host 5-8 us longer.
+// reads, 1423 and 1406 us; 512 steps of 96 instances of 256^2 6905 and 6925 us, of
+// 40 of 300^2 with Heun 10808 and 10921 (other register spills); 256 steps of 129
+// different grids of up to 311 x 149 1224 and 1240, of 300 such grids 2629 and
+// 2743.  The parameters stay below 4 KB: beyond that a launch takes the host 5-8
+// us longer.
 constexpr int kTileRuns = 224, kTileIndex = 64;
 struct TileRun {
     int first, tiles, place, across;

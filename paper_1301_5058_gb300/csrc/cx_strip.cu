@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(32)
 
 template <int LAW, int MOB, bool HEUN>
 __global__ void __launch_bounds__(32)
-    batch_strip_kernel(const InstDev<double> *__restrict__ inst,
-                       const __grid_constant__ TileRuns runs, int parity, int stages, int halo)
+    batch_strip_kernel(const InstDev<double> *__restrict__ inst, int parity, int stages, int halo,
+                       const __grid_constant__ TileRuns runs)
 {
     // the table is not written while a pass may be queued
     const batch::TileAt w = batch::tile_of_block(runs, blockIdx.x);
@@ -98,7 +98,7 @@ cudaError_t launch_v(const TileLaunch &a, const TilePlan &p, cudaStream_t st)
 {
     if (a.inst)
         return launch_pass(batch_strip_kernel<LAW, MOB, HEUN>, a.runs->run[a.runs->n].first, 32, 0, st,
-                           (const InstDev<double> *)a.inst, *a.runs, a.parity, p.stages(), p.halo_x());
+                           (const InstDev<double> *)a.inst, a.parity, p.stages(), p.halo_x(), *a.runs);
     const StepArgs &g = *a.grid;
     const Ptrs<double> P{(const double *)g.b, (const double *)g.n, (const double *)g.s, nullptr,
                          nullptr, (double *)g.bo, (double *)g.no};

@@ -53,9 +53,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 // One tile of an instance of a batch.
 template <int LAW, int MOB, int NOISE, bool HEUN, int LX, int R>
 __global__ void __launch_bounds__(kMaxThreads, 1)
-    batch_tile_kernel(const InstDev<float> *__restrict__ inst,
-                      const __grid_constant__ TileRuns runs, int parity, int steps,
-                      const long long *step_base, int step_off)
+    batch_tile_kernel(const InstDev<float> *__restrict__ inst, int parity, int steps,
+                      const long long *step_base, int step_off,
+                      const __grid_constant__ TileRuns runs)
 {
     // the table is not written while a pass may be queued
     const batch::TileAt w = batch::tile_of_block(runs, blockIdx.x);
@@ -82,8 +82,8 @@ cudaError_t launch_v(const TileLaunch &a, const TilePlan &p, cudaStream_t st)
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         return launch_pass(kern, a.runs->run[a.runs->n].first, p.threads, smem, st,
-                           (const InstDev<float> *)a.inst, *a.runs, a.parity, p.steps, a.nz.step_base,
-                           a.nz.step_off);
+                           (const InstDev<float> *)a.inst, a.parity, p.steps, a.nz.step_base,
+                           a.nz.step_off, *a.runs);
     }
     const StepArgs &g = *a.grid;
     const KV<float2> k = make_kv(coef_t<float>(g.k));
