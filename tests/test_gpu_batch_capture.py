@@ -56,7 +56,7 @@ def test_captured_steps_of_a_new_length(cx, kw, sizes):
         assert np.array_equal(b, want[0]) and np.array_equal(n, want[1])
 
 
-@pytest.mark.parametrize("count", [223, 224, 225, 600])
+@pytest.mark.parametrize("count", [8, 9, 20, 223, 224, 225, 600])
 @pytest.mark.parametrize("kw", [dict(), dict(noise_mode=1, noise_dist=1), dict(precision=0)],
                          ids=["tiles", "per-step", "strips"])
 def test_more_sizes_than_runs_of_a_launch(cx, kw, count):
@@ -68,7 +68,7 @@ def test_more_sizes_than_runs_of_a_launch(cx, kw, count):
     specs.append(dict(specs[5], seed=1000))  # a size of two instances
     with cx.Batch(specs) as bt:
         bt.step(64 + 9)
-        for i in [*range(0, count, count // 18), count - 1, 5, count]:
+        for i in [*range(0, count, max(1, count // 18)), count - 1, 5, count]:
             want = single_march(cx, specs[i], 64 + 9, dtype)
             assert np.array_equal(bt.field(i, cx.CX_FIELD_B, dtype), want[0]), i
             assert np.array_equal(bt.field(i, cx.CX_FIELD_N, dtype), want[1]), i
